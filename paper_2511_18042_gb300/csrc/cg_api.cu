@@ -334,6 +334,12 @@ static void fill_devgrid(const cg_grid* g, const cg_params* p, DevGrid& d) {
       d.cig[dir] = ig;
       d.cig2[dir] = 1.0 / g2;
       for (int m = 0; m < 3; ++m) { d.cn[dir][m] = n[m]; d.ct1[dir][m] = t1[m]; d.ct2[dir][m] = t2[m]; }
+      d.unit[dir] = 1;
+      for (int m = 0; m < nd; ++m) {
+        const double v[3] = {n[m], t1[m], t2[m]};
+        for (int k = 0; k < nd; ++k)
+          if (frame_nz(true, nd, dir, k, m) && fabs(v[k]) != 1.0) d.unit[dir] = 0;
+      }
     }
   }
   d.twall = p->twall;
@@ -684,6 +690,10 @@ static GbrCfg gbr_cfg(const cg_solver* s) {
   q.f_thr = (float)q.thr;
   q.f_eps = (float)q.eps;
   q.f_alpha = (float)q.alpha;
+  const double big = 0x1p400;
+  q.f64_fast = q.gm1 > 1.0 / big && q.gm1 < big && q.gamma > 1.0 / big && q.gamma < big && q.eps >= 0.0 && q.eps < big &&
+               fabs(q.alpha) < big;
+  q.d_gm1 = host_divisor(q.f64_fast ? q.gm1 : 1.0);
   return q;
 }
 

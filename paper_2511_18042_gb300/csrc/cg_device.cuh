@@ -36,6 +36,7 @@ struct DevGrid {
   // with the same operations as the per-interface frame of a curvilinear one)
   double cg2[3], cg[3], cig[3], cig2[3];
   double cn[3][3], ct1[3][3], ct2[3][3];
+  int unit[3];      // the frame's non-zero entries are exactly +1 or -1
   // curvilinear metrics: planes on the box padded by PM in active directions
   int P[3];
   long long NP;
@@ -398,6 +399,11 @@ __device__ __forceinline__ T d4(T m2, T m1, T p1, T p2) {
 template <typename T = double>
 __device__ __forceinline__ T d2_from_grad(T wm, T w0, T wp, T dm, T dp) {
   return T(2.0) * (wp - T(2.0) * w0 + wm) - T(0.5) * (dp - dm);
+}
+
+// half of it: the factors 2 and 1/2 are exact, so this rounds as d2_from_grad does
+__device__ __forceinline__ double d2_half_from_grad(double wm, double w0, double wp, double dm, double dp) {
+  return __fma_rn(-0.25, dp - dm, __fma_rn(-2.0, w0, wp) + wm);
 }
 
 // ---------------------------------------------------------------- MP5

@@ -3,6 +3,7 @@
 // Eq. (9)-(10), and the kernels of one RK stage.
 #pragma once
 #include "cg_device.cuh"
+#include "cg_fp64.cuh"
 
 namespace cgk {
 
@@ -10,6 +11,8 @@ struct GbrCfg {
   double gamma, gm1, thr, eps, alpha;
   int window;  // interface sensor window half-width
   float f_gamma, f_gm1, f_thr, f_eps, f_alpha;  // FP32 copies for the mixed form
+  Divisor d_gm1;     // gamma - 1 as a divisor (FP64 form)
+  int f64_fast;      // the parameters suit gbr_flux_f64
 };
 
 // interface frame: unit normal, tangents, averaged state and its sound speed
@@ -135,17 +138,17 @@ __device__ __forceinline__ void hllc(T gamma, T gm1, const T* WL, const T* WR, c
 }
 
 // Flux at one interface i+1/2 from the stencil W_{i-2..i+3}, the gradients
-// W'_{i,i+1}, second derivatives W''_{i,i+1}, the interface sensor and the
-// interface metrics.  Wave order: 0 = u_n - c, 1 = entropy, 2.. = shear,
+// W'_{i,i+1}, second derivatives W''_{i,i+1}, whether the interface's sensor is
+// above its threshold (disc) and the interface metrics.  Wave order: 0 = u_n - c, 1 = entropy, 2.. = shear,
 // last = u_n + c.
 template <int ND, bool CART, int DIR, typename T = double>
 __device__ __forceinline__ void gbr_flux(const GbrCfg& q, const DevGrid& g, const T (&Wst)[6][ND + 2],
-                                         const T (&Wd)[2][ND + 2], const T (&Wdd)[2][ND + 2], T omb,
+                                         const T (&Wd)[2][ND + 2], const T (&Wdd)[2][ND + 2], bool disc,
                                          const T* xi, T* F) {
   constexpr int NV = ND + 2, IP = ND + 1;
   const T c12 = T(1.0 / 12.0);
   const T gamma = gconst<T>(q.gamma, q.f_gamma), gm1 = gconst<T>(q.gm1, q.f_gm1),
-          alpha = gconst<T>(q.alpha, q.f_alpha), eps = gconst<T>(q.eps, q.f_eps), thr = gconst<T>(q.thr, q.f_thr);
+          alpha = gconst<T>(q.alpha, q.f_alpha), eps = gconst<T>(q.eps, q.f_eps);
   Frame<ND, T> fr;
   T g2, gg, ig2;
   if (CART) {
@@ -186,7 +189,6 @@ __device__ __forceinline__ void gbr_flux(const GbrCfg& q, const DevGrid& g, cons
     to_char<ND, CART, DIR, T>(fr, Wd[j], Cd[j]);
     to_char<ND, CART, DIR, T>(fr, Wdd[j], Cdd[j]);
   }
-  const bool disc = omb > thr;
   T CL[NV], CR[NV];
 #pragma unroll
   for (int b = 0; b < NV; ++b) {
@@ -234,6 +236,341 @@ __device__ __forceinline__ void gbr_flux(const GbrCfg& q, const DevGrid& g, cons
     for (int m = 0; m < ND; ++m) xl[m] = xi[m];
   }
   hllc<ND, CART, DIR, T>(gamma, gm1, WL, WR, xl, g2, gg, ig2, F);
+}
+
+// ---------------------------------------------------------------- FP64 form
+// The same flux in FP64, value for value what gbr_flux gives, with fewer
+// instructions on the FP64 pipe, which bounds the sweep (2 a clock an SM):
+//   * divisions and square roots on the integer and FP32 pipes (cg_fp64.cuh);
+//   * a product with a power of two is exact, so x - 2 y, x + y/2 and the like
+//     are one fused multiply-add, and the factor 2 of the second derivatives
+//     and of 1/c^2 = 2 (1/(2 c^2)) is carried along instead of multiplied;
+//   * comparisons, minima and minmods on the bit patterns;
+//   * the characteristic variables of the outer stencil nodes only where MP5
+//     reads them (the acoustic and shear waves of a flagged interface, the
+//     entropy wave where Eq. (8) limits it);
+//   * on a Cartesian grid whose unit normals are exactly 1 (UN) no
+//     multiplication by them.
+// Measured (triple point 1792 x 768, MEG6): FP64 instructions an interface 569
+// -> 272 (with the staging and the epilogue), FP64 pipe 80 % busy; the sweep
+// 1.51 -> 0.79 ms a launch, the whole step 9.98 -> 5.60 ms.
+// Returns false where an operand is out of the range of these forms (a state
+// that is not positive, NaN, extreme magnitudes): the caller then repeats the
+// interface with gbr_flux.
+// (mp5's value; the range tests of its operands go to R)
+__device__ __forceinline__ double mp5_f64(double um2, double um1, double u0, double up1, double up2, double alpha,
+                                          double eps, F64Range& R) {
+  // 60 = 1.875 2^5: B, 2^105 / B, 1 / 1.875 and the exponent word of div_by
+  const Divisor sixty{0x001e000000000000ull, 0x0011111111111111ull, 0.53333333333f, 0x40400000u};
+  double ul = __fma_rn(2.0, um2, -(13.0 * um1)) + 47.0 * u0 + 27.0 * up1 - 3.0 * up2;
+  R.any0(ul);
+  ul = div_by(ul, sixty);
+  const double dm = u0 - um1, dp = up1 - u0, adm = alpha * dm;
+  const double ump = u0 + minmod_f64(dp, adm);
+  if (bits64((ul - u0) * (ul - ump)) <= bits64(eps)) return ul;
+  const double dm1 = __fma_rn(-2.0, um1, um2) + u0;
+  const double d0 = __fma_rn(-2.0, u0, um1) + up1;
+  const double dp1 = __fma_rn(-2.0, up1, u0) + up2;
+  const double dm4p = minmod_f64(minmod_f64(__fma_rn(4.0, d0, -dp1), __fma_rn(4.0, dp1, -d0)), minmod_f64(d0, dp1));
+  const double dm4m = minmod_f64(minmod_f64(__fma_rn(4.0, d0, -dm1), __fma_rn(4.0, dm1, -d0)), minmod_f64(d0, dm1));
+  const double uul = u0 + adm;
+  const double umd = 0.5 * ((u0 + up1) - dm4p);
+  const double ulc = __fma_rn(0.5, dm, u0) + (4.0 / 3.0) * dm4m;
+  const long long k0 = order_key(u0), k1 = order_key(up1), kd = order_key(umd), kl = order_key(uul), kc = order_key(ulc);
+  const double umin = from_key(kmax(kmin(kmin(k0, k1), kd), kmin(kmin(k0, kl), kc)));
+  const double umax = from_key(kmin(kmax(kmax(k0, k1), kd), kmax(kmax(k0, kl), kc)));
+  return ul + minmod_f64(umin - ul, umax - ul);
+}
+
+// The left and right MP5 states of one wave from its stencil v0..v5: a
+// function of its own, so that the sweep holds its code once (few warps take
+// it, and inlined for every wave and side it would crowd the instruction cache).
+struct Mp5Pair {
+  double L, R;
+  unsigned worst;
+};
+static __device__ __noinline__ Mp5Pair mp5_pair_f64(double v0, double v1, double v2, double v3, double v4, double v5,
+                                                    double alpha, double eps) {
+  F64Range R;
+  Mp5Pair o;
+  o.L = mp5_f64(v0, v1, v2, v3, v4, alpha, eps, R);
+  o.R = mp5_f64(v5, v4, v3, v2, v1, alpha, eps, R);
+  o.worst = R.worst;
+  return o;
+}
+
+// characteristic variables of a primitive vector (to_char's values)
+template <int ND, bool CART, int DIR, bool UN>
+__device__ __forceinline__ void to_char_f64(const Frame<ND, double>& f, const double* w, double* c) {
+  constexpr int IP = ND + 1;
+  const double un = UN ? by_sign(f.n[DIR], w[1 + DIR]) : sdot<ND, CART, DIR, 0, double>(f.n, w + 1);
+  const double a = f.ha * w[IP], b = f.hb * un;
+  c[0] = a - b;
+  c[1] = __fma_rn(-2.0, a, w[0]);
+  c[IP] = a + b;
+#pragma unroll
+  for (int m = 0; m < ND; ++m) {
+    if (UN && ND >= 2 && frame_nz(CART, ND, DIR, 1, m)) c[2] = by_sign(f.t1[m], w[1 + m]);
+    if (UN && ND == 3 && frame_nz(CART, ND, DIR, 2, m)) c[3] = by_sign(f.t2[m], w[1 + m]);
+  }
+  if (!UN && ND >= 2) c[2] = sdot<ND, CART, DIR, 1, double>(f.t1, w + 1);
+  if (!UN && ND == 3) c[3] = sdot<ND, CART, DIR, 2, double>(f.t2, w + 1);
+}
+
+template <int ND, bool CART, int DIR, bool UN>
+__device__ __forceinline__ void from_char_f64(const Frame<ND, double>& f, double cb2, const double* c, double* w) {
+  constexpr int IP = ND + 1;
+  if (!UN) {
+    from_char<ND, CART, DIR, double>(f, c, w);
+    return;
+  }
+  const double s = c[0] + c[IP];
+  w[0] = c[1] + s;
+  w[IP] = cb2 * s;
+#pragma unroll
+  for (int m = 0; m < ND; ++m) {
+    if (m == DIR) w[1 + m] = by_sign(f.n[m], (c[IP] - c[0]) * f.cr);
+    else if (ND >= 2 && frame_nz(CART, ND, DIR, 1, m)) w[1 + m] = by_sign(f.t1[m], c[2]);
+    else w[1 + m] = by_sign(f.t2[m], c[3]);
+  }
+}
+
+template <int ND, bool CART, int DIR>
+__device__ __forceinline__ void hllc_f64(const GbrCfg& q, const double* WL, const double* WR, const double* xi,
+                                         double g2, double g, double ig2, double* F, F64Range& R) {
+  constexpr int IP = ND + 1;
+  const double rL = WL[0], pL = WL[IP], rR = WR[0], pR = WR[IP];
+  R.pos(rL);
+  R.pos(pL);
+  R.pos(rR);
+  R.pos(pR);
+  const double UL = sdot<ND, CART, DIR, 0, double>(xi, WL + 1);
+  const double UR = sdot<ND, CART, DIR, 0, double>(xi, WR + 1);
+  double SL, SR, EL, ER;
+  {
+    double qL = WL[1] * WL[1], qR = WR[1] * WR[1];
+#pragma unroll
+    for (int m = 1; m < ND; ++m) {
+      qL = qL + WL[1 + m] * WL[1 + m];
+      qR = qR + WR[1 + m] * WR[1 + m];
+    }
+    EL = __fma_rn(0.5, rL * qL, div_by(pL, q.d_gm1));
+    ER = __fma_rn(0.5, rR * qR, div_by(pR, q.d_gm1));
+    double cL, cR, HL, HR;
+    {
+      const Divisor D = divisor(rL);
+      const double HN = EL + pL;
+      R.any0(HN);
+      cL = sqrt_ranged(div_by(q.gamma * pL, D));
+      HL = div_by(HN, D);
+    }
+    {
+      const Divisor D = divisor(rR);
+      const double HN = ER + pR;
+      R.any0(HN);
+      cR = sqrt_ranged(div_by(q.gamma * pR, D));
+      HR = div_by(HN, D);
+    }
+    const double sL = sqrt_ranged(rL), sR = sqrt_ranged(rR);
+    const double iden = rcp_by(divisor(sL + sR));
+    double uh[3];
+#pragma unroll
+    for (int m = 0; m < ND; ++m) uh[m] = (sL * WL[1 + m] + sR * WR[1 + m]) * iden;
+    double qh = uh[0] * uh[0];
+#pragma unroll
+    for (int m = 1; m < ND; ++m) qh = qh + uh[m] * uh[m];
+    const double Uh = sdot<ND, CART, DIR, 0, double>(xi, uh);
+    const double Hh = (sL * HL + sR * HR) * iden;
+    const double c2 = q.gm1 * __fma_rn(-0.5, qh, Hh);
+    R.pos(c2);
+    const double chg = sqrt_ranged(c2) * g;
+    SL = min_f64(UL - cL * g, Uh - chg);
+    SR = max_f64(UR + cR * g, Uh + chg);
+  }
+  double Ss;
+  {
+    const double eR = SR - UR, eL = SL - UL;
+    const double num = rR * UR * eR - rL * UL * eL + (pL - pR) * g2, den = rR * eR - rL * eL;
+    R.any0(num);
+    R.any(den);
+    Ss = div_by(num, divisor(den));
+  }
+  const bool left = nonneg(SL) || nonneg(Ss);
+  const bool star = !nonneg(SL) && nonneg(SR);
+  double W[ND];
+#pragma unroll
+  for (int m = 0; m < ND; ++m) W[m] = left ? WL[1 + m] : WR[1 + m];
+  const double r = left ? rL : rR, p = left ? pL : pR, U = left ? UL : UR, E = left ? EL : ER, S = left ? SL : SR;
+  double ru[ND];
+  F[0] = r * U;
+#pragma unroll
+  for (int m = 0; m < ND; ++m) {
+    ru[m] = r * W[m];
+    F[1 + m] = frame_nz(CART, ND, DIR, 0, m) ? ru[m] * U + xi[m] * p : ru[m] * U;
+  }
+  F[IP] = (E + p) * U;
+  if (!star) return;
+  const double SU = S - U, rSU = r * SU, SS = S - Ss, d = Ss - U;
+  R.any(rSU);
+  R.any(SS);
+  R.any0(E);
+  const double fac = div_by(rSU, divisor(SS));
+  F[0] = F[0] + S * (fac - r);
+#pragma unroll
+  for (int m = 0; m < ND; ++m) {
+    const double qs = frame_nz(CART, ND, DIR, 0, m) ? fac * (W[m] + xi[m] * d * ig2) : fac * W[m];
+    F[1 + m] = F[1 + m] + S * (qs - ru[m]);
+  }
+  const double qe = fac * (div_by(E, divisor(r)) + d * (Ss * ig2 + div_by(p, divisor(rSU))));
+  F[IP] = F[IP] + S * (qe - E);
+}
+
+// W(j, w): the primitives of stencil node i-2+j (j = 0..5); Wd(j, w), Wh(j, w):
+// first derivatives and halved second derivatives of node i+j (j = 0, 1).
+template <int ND, bool CART, int DIR, bool UN, class FW, class FD, class FH>
+__device__ __forceinline__ bool gbr_flux_f64(const GbrCfg& q, const DevGrid& g, FW ldW, FD ldD, FH ldH, bool disc,
+                                             const double* xi, double* F) {
+  constexpr int NV = ND + 2, IP = ND + 1;
+  F64Range R;
+  if (!q.f64_fast) R.see(~0u);
+  Frame<ND, double> fr;
+  double g2, gg, ig2, xl[3];
+  if (CART) {
+    g2 = g.cg2[DIR];
+    gg = g.cg[DIR];
+    ig2 = g.cig2[DIR];
+#pragma unroll
+    for (int m = 0; m < ND; ++m) {
+      fr.n[m] = g.cn[DIR][m];
+      fr.t1[m] = g.ct1[DIR][m];
+      fr.t2[m] = g.ct2[DIR][m];
+      xl[m] = m == DIR ? g.cxh[DIR] : 0.0;
+    }
+  } else {
+#pragma unroll
+    for (int m = 0; m < ND; ++m) xl[m] = xi[m];
+    g2 = xi[0] * xi[0];
+#pragma unroll
+    for (int m = 1; m < ND; ++m) g2 = g2 + xi[m] * xi[m];
+    R.pos(g2);
+    gg = sqrt_ranged(g2);
+    const double ig = rcp_by(divisor(gg));
+    ig2 = rcp_by(divisor(g2));
+#pragma unroll
+    for (int m = 0; m < ND; ++m) fr.n[m] = xi[m] * ig;
+    if (ND == 2) {
+      fr.t1[0] = -fr.n[1];
+      fr.t1[1] = fr.n[0];
+    } else if (ND == 3) {  // tangents(): t1 from the two largest components of n, t2 = n x t1
+      const double* n = fr.n;
+      int s = 0;
+      if (order_key(fabs(n[1])) < order_key(fabs(n[0]))) s = 1;
+      if (order_key(fabs(n[2])) < order_key(fabs(s == 1 ? n[1] : n[0]))) s = 2;
+      const double na = s == 0 ? n[1] : (s == 1 ? n[2] : n[0]), nb = s == 0 ? n[2] : (s == 1 ? n[0] : n[1]);
+      const double r = rcp_by(divisor(sqrt_ranged(na * na + nb * nb)));
+      const double ta = -nb * r, tb = na * r;
+      fr.t1[0] = s == 0 ? 0.0 : (s == 1 ? tb : ta);
+      fr.t1[1] = s == 0 ? ta : (s == 1 ? 0.0 : tb);
+      fr.t1[2] = s == 0 ? tb : (s == 1 ? ta : 0.0);
+      fr.t2[0] = n[1] * fr.t1[2] - n[2] * fr.t1[1];
+      fr.t2[1] = n[2] * fr.t1[0] - n[0] * fr.t1[2];
+      fr.t2[2] = n[0] * fr.t1[1] - n[1] * fr.t1[0];
+    }
+  }
+  double w2[NV], w3[NV];
+  ldW(2, w2);
+  ldW(3, w3);
+  double cb2;
+  {
+    const double rs = w2[0] + w3[0], ps = w2[IP] + w3[IP];  // twice the averaged density and pressure
+    R.pos(rs);
+    R.pos(ps);
+    const Divisor D = divisor(rs);
+    fr.cb = sqrt_ranged(div_by(q.gamma * ps, D));
+    const double ic = rcp_by(divisor(fr.cb));
+    fr.ic2 = ic * ic;
+    fr.ha = scale2<-1>(fr.ic2);
+    fr.hb = scale2<-2>(rs * ic);
+    fr.cr = scale2<1>(div_by(fr.cb, D));
+    cb2 = fr.cb * fr.cb;
+  }
+  double CL[NV], CR[NV], C2[NV], C3[NV];
+  to_char_f64<ND, CART, DIR, UN>(fr, w2, C2);
+  to_char_f64<ND, CART, DIR, UN>(fr, w3, C3);
+  const double c6 = 2.0 * (1.0 / 12.0);
+  {
+    double w[NV], c[NV];
+    ldD(0, w);
+    to_char_f64<ND, CART, DIR, UN>(fr, w, c);
+#pragma unroll
+    for (int b = 0; b < NV; ++b) CL[b] = __fma_rn(0.5, c[b], C2[b]);
+    ldH(0, w);
+    to_char_f64<ND, CART, DIR, UN>(fr, w, c);
+#pragma unroll
+    for (int b = 0; b < NV; ++b) CL[b] = CL[b] + c[b] * c6;
+    ldD(1, w);
+    to_char_f64<ND, CART, DIR, UN>(fr, w, c);
+#pragma unroll
+    for (int b = 0; b < NV; ++b) CR[b] = __fma_rn(-0.5, c[b], C3[b]);
+    ldH(1, w);
+    to_char_f64<ND, CART, DIR, UN>(fr, w, c);
+#pragma unroll
+    for (int b = 0; b < NV; ++b) CR[b] = CR[b] + c[b] * c6;
+  }
+  {  // entropy wave: MP criterion
+    auto entropy = [&](int j) {
+      double w[NV];
+      ldW(j, w);
+      return __fma_rn(-2.0, fr.ha * w[IP], w[0]);
+    };
+    const double v1 = entropy(1), v2 = C2[1], v3 = C3[1], v4 = entropy(4);
+    const double cl = CL[1], cr = CR[1], cc = 0.5 * (cl + cr), dv = v3 - v2;
+    const double umpL = v2 + minmod_f64(dv, q.alpha * (v2 - v1));
+    const double umpR = v3 + minmod_f64(-dv, q.alpha * (v3 - v4));
+    const double tL = (cl - v2) * (cl - umpL), tR = (cr - v3) * (cr - umpR);
+    // finite and above eps
+    const bool limL = bits64(tL) > bits64(q.eps) && __double2hiint(tL) < 0x7ff00000;
+    const bool limR = bits64(tR) > bits64(q.eps) && __double2hiint(tR) < 0x7ff00000;
+    CL[1] = cc;
+    CR[1] = cc;
+    if (limL || limR) {
+      const Mp5Pair m = mp5_pair_f64(entropy(0), v1, v2, v3, v4, entropy(5), q.alpha, q.eps);
+      R.see(m.worst);
+      if (limL) CL[1] = m.L;
+      if (limR) CR[1] = m.R;
+    }
+  }
+  if (!disc) {  // acoustic waves upwind, shear waves central
+#pragma unroll
+    for (int b = 2; b < IP; ++b) {
+      const double cc = 0.5 * (CL[b] + CR[b]);
+      CL[b] = cc;
+      CR[b] = cc;
+    }
+  } else {
+    double C0[NV], C1[NV], C4[NV], C5[NV], w[NV];
+    ldW(0, w);
+    to_char_f64<ND, CART, DIR, UN>(fr, w, C0);
+    ldW(1, w);
+    to_char_f64<ND, CART, DIR, UN>(fr, w, C1);
+    ldW(4, w);
+    to_char_f64<ND, CART, DIR, UN>(fr, w, C4);
+    ldW(5, w);
+    to_char_f64<ND, CART, DIR, UN>(fr, w, C5);
+#pragma unroll
+    for (int b = 0; b < NV; ++b) {
+      if (b == 1) continue;
+      const Mp5Pair m = mp5_pair_f64(C0[b], C1[b], C2[b], C3[b], C4[b], C5[b], q.alpha, q.eps);
+      R.see(m.worst);
+      CL[b] = m.L;
+      CR[b] = m.R;
+    }
+  }
+  double WL[NV], WR[NV];
+  from_char_f64<ND, CART, DIR, UN>(fr, cb2, CL, WL);
+  from_char_f64<ND, CART, DIR, UN>(fr, cb2, CR, WR);
+  hllc_f64<ND, CART, DIR>(q, WL, WR, xl, g2, gg, ig2, F, R);
+  return R.ok();
 }
 
 }  // namespace cgk

@@ -473,7 +473,7 @@ constexpr int SWEEP_TL = 64;
 __host__ __device__ constexpr int sweep_lw(int dir) { return dir == 0 ? 4 : 8; }
 template <int ND, int LW>
 __host__ __device__ constexpr int sweep_smem_doubles() {
-  return (ND + 2) * (SWEEP_TL + 9 + SWEEP_TL + 3 + SWEEP_TL + 1 + SWEEP_TL) * LW + (SWEEP_TL + 7) * LW;
+  return (ND + 2) * (SWEEP_TL + 9 + SWEEP_TL + 3 + SWEEP_TL + 1 + SWEEP_TL) * LW;
 }
 
 // Blocks per SM the register budget is sized for (256 threads a block):
@@ -496,7 +496,34 @@ __host__ __device__ constexpr int sweep_min_blocks() {
 // contraction, the oracle's operation order; 1: FP64 with fused multiply-add;
 // 2: FP32): the code is the same, the compilation flags differ, and distinct
 // instantiations keep the units' kernels apart.
-template <int ND, int DIR, bool CART, bool COMPACT, typename T, int LW, int UNIT>
+// The IEEE form of one interface flux of the FP64 sweep, from the staged tile:
+// the interfaces whose operands gbr_flux_f64 refuses.
+// io: the interface metrics in, the flux out.
+template <int ND, bool CART, int DIR, int LW>
+static __device__ __noinline__ void gbr_flux_ieee(const GbrCfg& q, const DevGrid& g, const double* sW, const double* sD,
+                                                  const double* sH, int a, int l, bool disc, double* io) {
+  constexpr int NV = ND + 2, RW = SWEEP_TL + 9, RD = SWEEP_TL + 3, RDD = SWEEP_TL + 1;
+  auto IX = [](int v, int r, int l_, int rows) {
+    return DIR == 0 ? (v * LW + l_) * rows + r : (v * rows + r) * LW + l_;
+  };
+  double Wst[6][NV], Wd[2][NV], Wdd[2][NV], F[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+#pragma unroll
+    for (int j = 0; j < 6; ++j) Wst[j][v] = sW[IX(v, a + 2 + j, l, RW)];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      Wd[j][v] = sD[IX(v, a + 1 + j, l, RD)];
+      Wdd[j][v] = 2.0 * sH[IX(v, a + j, l, RDD)];
+    }
+  }
+  const double xi[3] = {io[0], io[1], io[2]};
+  gbr_flux<ND, CART, DIR, double>(q, g, Wst, Wd, Wdd, disc, xi, F);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) io[v] = F[v];
+}
+
+template <int ND, int DIR, bool CART, bool COMPACT, typename T, int LW, int UNIT, bool UN = false>
 __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid& g, const GbrCfg& q, const StageArgs& A) {
   static_assert((SWEEP_TL * LW) % 256 == 0, "a tile must hold a multiple of the block's threads");
   constexpr int NV = ND + 2;
@@ -509,7 +536,6 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
   T* sD = sW + NV * RW * LW;
   T* sDD = sD + NV * RD * LW;
   T* sF = sDD + NV * RDD * LW;
-  T* sO = sF + NV * TL * LW;
   auto IX = [](int v, int r, int l, int rows) {
     return DIR == 0 ? (v * LW + l) * rows + r : (v * rows + r) * LW + l;
   };
@@ -560,6 +586,12 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
   // sensor box; node x of the line is at base + x * stride.
   __shared__ int s_lc[LW][3];
   __shared__ long long s_lq[LW], s_lo[LW];
+  // the line's nodes whose sensor is above the threshold, one bit a node (row
+  // r of the sensor window in bit r): an interface's maximum over its window is
+  // above the threshold where any bit of the window is set
+  __shared__ unsigned s_om[LW][4];
+  static_assert(RO <= 96, "three words of node bits and one read past them");
+  if (tid < LW * 4) s_om[tid >> 2][tid & 3] = 0u;
   if (tid < LW) {
     const int l = tid;
     int c[3] = {0, 0, 0};
@@ -640,14 +672,14 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
       }
       stn(sW, r, l, RW, w);
     }
-    // sensor window values
+    // sensor window: nodes above the threshold
+    const T thr = gconst<T>(q.thr, q.f_thr);
     for (int e = tid; e < RO * LW; e += blockDim.x) {
       int r = DIR == 0 ? e % RO : e / LW;
       int l = DIR == 0 ? e / RO : e % LW;
-      T o = T(0);
       int x = i0 - 4 + r;
-      if (s_lc[l][0] >= 0 && x <= n + 3) o = static_cast<const T*>(A.om)[s_lo[l] + (long long)x * os];
-      sO[(DIR == 0) ? l * RO + r : r * LW + l] = o;
+      if (s_lc[l][0] >= 0 && x <= n + 3 && static_cast<const T*>(A.om)[s_lo[l] + (long long)x * os] > thr)
+        atomicOr(&s_om[l][r >> 5], 1u << (r & 31));
     }
     __syncthreads();
     // 2. first derivatives along DIR on nodes i0-2 .. i0+TL
@@ -687,7 +719,10 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
       ldn(sD, r, l, RD, dm);
       ldn(sD, r + 2, l, RD, dp);
 #pragma unroll
-      for (int v = 0; v < NV; ++v) dd[v] = d2_from_grad(wm[v], w0[v], wp[v], dm[v], dp[v]);
+      for (int v = 0; v < NV; ++v) {
+        if constexpr (MIX) dd[v] = d2_from_grad(wm[v], w0[v], wp[v], dm[v], dp[v]);
+        else dd[v] = d2_half_from_grad(wm[v], w0[v], wp[v], dm[v], dp[v]);  // halved (gbr_flux_f64)
+      }
       stn(sDD, r, l, RDD, dd);
     }
     __syncthreads();
@@ -711,26 +746,38 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
       use_gbr = A.mask[A.tBox.at(c[0], c[1], c[2])] != 0 || A.mask[A.tBox.at(cn[0], cn[1], cn[2])] != 0;
     }
     if (use_gbr) {
-      T Wst[6][NV], Wd[2][NV], Wdd[2][NV];
-#pragma unroll
-      for (int j = 0; j < 6; ++j) ldn(sW, a + 2 + j, l, RW, Wst[j]);
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        ldn(sD, a + 1 + j, l, RD, Wd[j]);
-        ldn(sDD, a + j, l, RDD, Wdd[j]);
-      }
-      T omb = sO[(DIR == 0) ? l * RO + a + 3 : (a + 3) * LW + l];
-      for (int jj = 1 - q.window; jj <= q.window; ++jj) {
-        T o = sO[(DIR == 0) ? l * RO + a + 3 + jj : (a + 3 + jj) * LW + l];
-        omb = dmax(omb, o);
-      }
+      // nodes i-w+1 .. i+w of the sensor window, w = q.window <= 4
+      const int p0 = a + 4 - q.window;
+      const unsigned wb = __funnelshift_r(s_om[l][p0 >> 5], s_om[l][(p0 >> 5) + 1], p0 & 31);
+      const bool disc = (wb & ((1u << (2 * q.window)) - 1u)) != 0u;
       T xi[3] = {T(0), T(0), T(0)};
       if (!CART) {
         long long pq = plin(g, c[0], c[1], c[2]);
 #pragma unroll
         for (int m = 0; m < ND; ++m) xi[m] = to_t<T>(g.xt[(DIR * ND + m) * g.NP + pq]);
       }
-      gbr_flux<ND, CART, DIR, T>(q, g, Wst, Wd, Wdd, omb, xi, F);
+      if constexpr (MIX) {
+        T Wst[6][NV], Wd[2][NV], Wdd[2][NV];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) ldn(sW, a + 2 + j, l, RW, Wst[j]);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          ldn(sD, a + 1 + j, l, RD, Wd[j]);
+          ldn(sDD, a + j, l, RDD, Wdd[j]);
+        }
+        gbr_flux<ND, CART, DIR, T>(q, g, Wst, Wd, Wdd, disc, xi, F);
+      } else {
+        const bool good = gbr_flux_f64<ND, CART, DIR, UN>(
+            q, g, [&](int j, double* w) { ldn(sW, a + 2 + j, l, RW, w); },
+            [&](int j, double* w) { ldn(sD, a + 1 + j, l, RD, w); }, [&](int j, double* w) { ldn(sDD, a + j, l, RDD, w); },
+            disc, xi, F);
+        if (!good) {
+          double io[5] = {xi[0], xi[1], xi[2], 0.0, 0.0};
+          gbr_flux_ieee<ND, CART, DIR, LW>(q, g, sW, sD, sDD, a, l, disc, io);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) F[v] = io[v];
+        }
+      }
     } else if (ok) {
       long long hi = A.hBox.at(c[0], c[1], c[2]);
       long long hs = A.hBox.size();
@@ -784,9 +831,10 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
   }
 }
 
-template <int ND, int DIR, bool CART, bool COMPACT, typename T, int LW, int UNIT>
-__global__ void __launch_bounds__(256, sweep_min_blocks<ND, CART, T>()) k_gbr_sweep(DevGrid g, GbrCfg q, StageArgs A) {
-  k_gbr_sweep_body<ND, DIR, CART, COMPACT, T, LW, UNIT>(hw_block(), g, q, A);
+template <int ND, int DIR, bool CART, bool COMPACT, typename T, int LW, int UNIT, bool UN>
+__global__ void __launch_bounds__(256, sweep_min_blocks<ND, CART, T>())
+    k_gbr_sweep(const __grid_constant__ DevGrid g, const __grid_constant__ GbrCfg q, const __grid_constant__ StageArgs A) {
+  k_gbr_sweep_body<ND, DIR, CART, COMPACT, T, LW, UNIT, UN>(hw_block(), g, q, A);
 }
 
 // ---------------------------------------------------------------- deferred stage update

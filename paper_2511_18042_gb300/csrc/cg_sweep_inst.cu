@@ -30,18 +30,28 @@ dim3 sweep_grid(const DevGrid& g) {
   return sweep_grid_dims(DIR, LW, g);
 }
 
-template <int DIR, bool CART, bool COMPACT, int LW>
-int launch_one(const DevGrid& g, const GbrCfg& q, const StageArgs& A, cudaStream_t st) {
+template <int DIR, bool CART, bool COMPACT, int LW, bool UN>
+int launch_form(const DevGrid& g, const GbrCfg& q, const StageArgs& A, cudaStream_t st) {
   size_t smem = sizeof(ST) * sweep_smem_doubles<SND, LW>();
+  auto* k = k_gbr_sweep<SND, DIR, CART, COMPACT, ST, LW, CGK_SWEEP_UNIT, UN>;
   static bool attr_set = false;
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_gbr_sweep<SND, DIR, CART, COMPACT, ST, LW, CGK_SWEEP_UNIT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     attr_set = true;
   }
-  k_gbr_sweep<SND, DIR, CART, COMPACT, ST, LW, CGK_SWEEP_UNIT><<<sweep_grid<DIR, LW>(g), 256, smem, st>>>(g, q, A);
+  k<<<sweep_grid<DIR, LW>(g), 256, smem, st>>>(g, q, A);
   return (int)cudaGetLastError();
+}
+
+// FP64 on a Cartesian grid whose frame is exactly +-1: the form without the
+// multiplications by it.
+template <int DIR, bool CART, bool COMPACT, int LW>
+int launch_one(const DevGrid& g, const GbrCfg& q, const StageArgs& A, cudaStream_t st) {
+  if constexpr (CART && sizeof(ST) == 8) {
+    if (g.unit[DIR]) return launch_form<DIR, CART, COMPACT, LW, true>(g, q, A, st);
+  }
+  return launch_form<DIR, CART, COMPACT, LW, false>(g, q, A, st);
 }
 
 template <int DIR, int LW>
@@ -55,7 +65,9 @@ int launch_dir(int lw, bool cart, bool compact, const DevGrid& g, const GbrCfg& 
                cudaStream_t st) {
   if (lw == 4) return launch_kind<DIR, 4>(cart, compact, g, q, A, st);
   if (lw == 8) return launch_kind<DIR, 8>(cart, compact, g, q, A, st);
-  if (DIR > 0 && lw == 16) return launch_kind<DIR, 16>(cart, compact, g, q, A, st);
+  if constexpr (DIR > 0) {
+    if (lw == 16) return launch_kind<DIR, 16>(cart, compact, g, q, A, st);
+  }
   return (int)cudaErrorInvalidValue;
 }
 
