@@ -11,6 +11,7 @@
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
+#include "cg_fp64.cuh"
 
 namespace cgk {
 
@@ -165,13 +166,13 @@ __device__ __forceinline__ void prim_to_cons(const DevGrid& g, const double* W, 
     Q[1 + k] = W[0] * W[1 + k];
     q = q + W[1 + k] * W[1 + k];
   }
-  Q[ND + 1] = W[ND + 1] / g.gm1 + 0.5 * W[0] * q;
+  Q[ND + 1] = add_scaled(div_f64(W[ND + 1], g.gm1), 0.5, W[0] * q);
 }
 
 template <int ND>
 __device__ __forceinline__ void cons_to_prim_g(const DevGrid& g, const double* Q, double* W) {
   double rho = Q[0];
-  double irho = 1.0 / rho;
+  double irho = rcp_f64(rho);
   double ke = 0.0;
   W[0] = rho;
 #pragma unroll
@@ -179,7 +180,7 @@ __device__ __forceinline__ void cons_to_prim_g(const DevGrid& g, const double* Q
     W[1 + k] = Q[1 + k] * irho;
     ke = ke + Q[1 + k] * W[1 + k];
   }
-  W[ND + 1] = g.gm1 * (Q[ND + 1] - 0.5 * ke);
+  W[ND + 1] = g.gm1 * add_scaled(Q[ND + 1], -0.5, ke);
 }
 
 // ---------------------------------------------------------------- binary64 <-> binary32
@@ -263,9 +264,9 @@ __device__ __forceinline__ void cons_to_prim_mixed(double gm1, const double* Q, 
 template <int ND, typename T = double>
 __device__ __forceinline__ void wall_image(const DevGrid& g, T* w) {
   constexpr int IP = ND + 1;
-  T Tm = T(g.gm2) * w[IP] / w[0];
+  T Tm = div_t(T(g.gm2) * w[IP], w[0]);
   T Tg = T(2.0) * T(g.twall) - Tm;
-  w[0] = T(g.gm2) * w[IP] / Tg;
+  w[0] = div_t(T(g.gm2) * w[IP], Tg);
 #pragma unroll
   for (int m = 0; m < ND; ++m) w[1 + m] = -w[1 + m];
 }
@@ -368,7 +369,7 @@ struct LineBuf {
 template <int ND>
 __device__ __forceinline__ void cons_to_prim(double gm1, const double* Q, double* W) {
   double rho = Q[0];
-  double irho = 1.0 / rho;
+  double irho = rcp_f64(rho);
   W[0] = rho;
   double ke = 0.0;
 #pragma unroll
@@ -376,7 +377,7 @@ __device__ __forceinline__ void cons_to_prim(double gm1, const double* Q, double
     W[1 + k] = Q[1 + k] * irho;
     ke = (k == 0) ? Q[1] * W[1] : ke + Q[1 + k] * W[1 + k];
   }
-  W[ND + 1] = gm1 * (Q[ND + 1] - 0.5 * ke);
+  W[ND + 1] = gm1 * add_scaled(Q[ND + 1], -0.5, ke);
 }
 
 // fused multiply-add in the arithmetic type

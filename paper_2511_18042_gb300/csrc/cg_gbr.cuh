@@ -3,7 +3,6 @@
 // Eq. (9)-(10), and the kernels of one RK stage.
 #pragma once
 #include "cg_device.cuh"
-#include "cg_fp64.cuh"
 
 namespace cgk {
 

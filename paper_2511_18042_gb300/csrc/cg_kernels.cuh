@@ -115,29 +115,50 @@ __device__ __forceinline__ void stage_epilogue(const DevGrid& g, const StageArgs
     }
     return;
   }
-  const double ca = A.stage == 2 ? 0.75 : (1.0 / 3.0), cb = A.stage == 2 ? 0.25 : (2.0 / 3.0);
   [[maybe_unused]] float cJf = 0.f;
   if constexpr (MIX) cJf = -((A.stage == 2 ? 0.25f : (2.0f / 3.0f)) * d2f_int(dt)) * d2f_int(J);
+  if (A.stage == 2) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const double un = A.Un[v * g.N + qi], uc = A.Uc[v * g.N + qi];
+      if constexpr (MIX) {
+        out[v] = __fma_rn(0.75, un, __fma_rn(0.25, uc, f2d_int(cJf * tot[v])));
+      } else {
+        const double r = -(J * wide(tot[v]));
+        out[v] = add_scaled(0.75 * un, 0.25, uc + dt * r);  // the product with 1/4 is exact
+      }
+      A.Uout[v * g.N + qi] = out[v];
+    }
+    return;
+  }
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     const double un = A.Un[v * g.N + qi], uc = A.Uc[v * g.N + qi];
     if constexpr (MIX) {
-      out[v] = __fma_rn(ca, un, __fma_rn(cb, uc, f2d_int(cJf * tot[v])));
+      out[v] = __fma_rn(1.0 / 3.0, un, __fma_rn(2.0 / 3.0, uc, f2d_int(cJf * tot[v])));
     } else {
       const double r = -(J * wide(tot[v]));
-      out[v] = ca * un + cb * (uc + dt * r);
+      out[v] = (1.0 / 3.0) * un + (2.0 / 3.0) * (uc + dt * r);
     }
     A.Uout[v * g.N + qi] = out[v];
   }
-  if (A.stage != 3) return;
   bool bad;
   if constexpr (MIX) {
     bad = mixed_nonphysical<ND>(out);
   } else {
-    double ke = out[1] * (out[1] / out[0]);
+    F64Range R;
+    R.pos(out[0]);
 #pragma unroll
-    for (int m = 1; m < ND; ++m) ke = ke + out[1 + m] * (out[1 + m] / out[0]);
-    double p = g.gm1 * (out[IP] - 0.5 * ke);
+    for (int m = 0; m < ND; ++m) R.any0(out[1 + m]);
+    const bool fast = R.ok();
+    const Divisor D = divisor(out[0]);
+    double ke = 0.0;
+#pragma unroll
+    for (int m = 0; m < ND; ++m) {
+      const double u = fast ? div_by(out[1 + m], D) : div_ieee(out[1 + m], out[0]);
+      ke = m == 0 ? out[1] * u : ke + out[1 + m] * u;
+    }
+    double p = g.gm1 * add_scaled(out[IP], -0.5, ke);
     bad = !(out[0] > 0.0) || !(p > 0.0);
   }
   if (bad) {
@@ -191,13 +212,19 @@ __global__ void k_prim(DevGrid g, const double* __restrict__ U, TW* __restrict__
 }
 
 // ---------------------------------------------------------------- sensor
-// Quotient of the sensor's ratios: IEEE division in FP64; in the mixed form's
+// Quotient of the sensor's ratios: correctly rounded in FP64; in the mixed form's
 // FP32 sensor the fast reciprocal-multiply (2 ulp, denominators below 2^126:
 // sums of pressures and of squared velocity gradients).
 template <typename T>
 __device__ __forceinline__ T sensor_div(T a, T b) {
   if constexpr (sizeof(T) == 4) return __fdividef(a, b);
-  else return a / b;
+  else return div_f64(a, b);
+}
+
+// Normalised pressure second difference of a node and its two neighbours.
+template <typename T>
+__device__ __forceinline__ T sensor_phi(T pm, T p0, T pp) {
+  return sensor_div(fabs(add_scaled(pp, T(-2.0), p0) + pm), add_scaled(pp, T(2.0), p0) + pm);
 }
 
 // Omega^d = phi * zeta on the box [-4, n+3]: phi the largest normalised
@@ -293,8 +320,7 @@ __device__ __forceinline__ void k_omega_body(const VBlock& vb, const DevGrid& g,
         const long long st = l == 0 ? 1 : (l == 1 ? (long long)g.n[0] : (long long)g.n[0] * g.n[1]);
         const T* P = W + IP * g.N + q;
         const T pm = T(P[-st]), pp = T(P[st]);
-        T a = sensor_div(fabs(pp - T(2.0) * p0 + pm), pp + T(2.0) * p0 + pm);
-        if (a > phi) phi = a;
+        phi = raise_to(phi, sensor_phi<T>(pm, p0, pp));
         if (!COMPACT) {
 #pragma unroll
           for (int k = 0; k < ND; ++k) {
@@ -327,8 +353,7 @@ __device__ __forceinline__ void k_omega_body(const VBlock& vb, const DevGrid& g,
         load_state<ND, false, T, T>(g, W, a[0], a[1], a[2], s[t]);
       }
       const T pm = T(s[2][IP]), pp = T(s[3][IP]);
-      T a = sensor_div(fabs(pp - T(2.0) * p0 + pm), pp + T(2.0) * p0 + pm);
-      if (a > phi) phi = a;
+      phi = raise_to(phi, sensor_phi<T>(pm, p0, pp));
       if (!COMPACT) {
 #pragma unroll
         for (int k = 0; k < ND; ++k)
@@ -401,8 +426,7 @@ __global__ void __launch_bounds__(OMT_X * OMT_Y) k_omega_tile(DevGrid g, const T
   T du[3][3];
   {  // x
     const T pm = sP[ty][tx - 1], pp = sP[ty][tx + 1];
-    T a = sensor_div(fabs(pp - T(2.0) * p0 + pm), pp + T(2.0) * p0 + pm);
-    if (a > phi) phi = a;
+    phi = raise_to(phi, sensor_phi<T>(pm, p0, pp));
 #pragma unroll
     for (int k = 0; k < ND; ++k)
       du[0][k] = d6<T>(sU[k][ty][tx - 3], sU[k][ty][tx - 2], sU[k][ty][tx - 1], sU[k][ty][tx + 1], sU[k][ty][tx + 2],
@@ -410,8 +434,7 @@ __global__ void __launch_bounds__(OMT_X * OMT_Y) k_omega_tile(DevGrid g, const T
   }
   {  // y
     const T pm = sP[ty - 1][tx], pp = sP[ty + 1][tx];
-    T a = sensor_div(fabs(pp - T(2.0) * p0 + pm), pp + T(2.0) * p0 + pm);
-    if (a > phi) phi = a;
+    phi = raise_to(phi, sensor_phi<T>(pm, p0, pp));
 #pragma unroll
     for (int k = 0; k < ND; ++k)
       du[1][k] = d6<T>(sU[k][ty - 3][tx], sU[k][ty - 2][tx], sU[k][ty - 1][tx], sU[k][ty + 1][tx], sU[k][ty + 2][tx],
@@ -433,8 +456,7 @@ __global__ void __launch_bounds__(OMT_X * OMT_Y) k_omega_tile(DevGrid g, const T
       for (int t = 0; t < 6; ++t) load_state<ND, false, T, T>(g, W, c[0], c[1], c[2] + (t < 3 ? t - 3 : t - 2), s[t]);
     }
     const T pm = s[2][IP], pp = s[3][IP];
-    T a = sensor_div(fabs(pp - T(2.0) * p0 + pm), pp + T(2.0) * p0 + pm);
-    if (a > phi) phi = a;
+    phi = raise_to(phi, sensor_phi<T>(pm, p0, pp));
 #pragma unroll
     for (int k = 0; k < ND; ++k)
       du[2][k] = d6<T>(s[0][1 + k], s[1][1 + k], s[2][1 + k], s[3][1 + k], s[4][1 + k], s[5][1 + k]);
@@ -909,7 +931,7 @@ __global__ void __launch_bounds__(256, 6) k_stage_update(DevGrid g, StageArgs A,
 template <int ND, bool CART, typename T>
 __device__ __forceinline__ T cfl_rate(const DevGrid& g, long long q, const T* w) {
   constexpr int IP = ND + 1;
-  T cs = sqrt(gconst<T>(g.gamma, g.f_gamma) * T(w[IP]) / T(w[0]));
+  T cs = sqrt_t(div_t(gconst<T>(g.gamma, g.f_gamma) * T(w[IP]), T(w[0])));
   T s = T(0);
   T J;
   if (CART) {
@@ -917,7 +939,7 @@ __device__ __forceinline__ T cfl_rate(const DevGrid& g, long long q, const T* w)
 #pragma unroll
     for (int l = 0; l < ND; ++l) {
       const T xh = gconst<T>(g.cxh[l], g.f_cxh[l]);
-      T t = fabs(xh * T(w[1 + l])) + cs * sqrt(xh * xh);
+      T t = fabs(xh * T(w[1 + l])) + cs * fabs(xh);  // |xi_hat_l| = sqrt(xh xh), the same value
       s = (l == 0) ? t : s + t;
     }
   } else {
@@ -934,7 +956,7 @@ __device__ __forceinline__ T cfl_rate(const DevGrid& g, long long q, const T* w)
         dot = (m == 0) ? x * T(w[1 + m]) : dot + x * T(w[1 + m]);
         mag = (m == 0) ? x * x : mag + x * x;
       }
-      T t = fabs(dot) + cs * sqrt(mag);
+      T t = fabs(dot) + cs * sqrt_t(mag);
       s = (l == 0) ? t : s + t;
     }
   }
@@ -974,7 +996,7 @@ __device__ __forceinline__ void k_cfl_max_body(const VBlock& vb, const DevGrid& 
       cons_to_prim<ND>(g.gm1, Q, w);
     }
     T r = cfl_rate<ND, CART, T>(g, q, w);
-    if (r > best) best = r;
+    best = raise_to(best, r);
   }
   cfl_block_max<T>(best, mx);
 }
@@ -1000,7 +1022,7 @@ __global__ void k_prim_cfl(DevGrid g, const double* __restrict__ U, TW* __restri
 #pragma unroll
     for (int v = 0; v < NV; ++v) W[v * g.N + q] = w[v];
     TW r = cfl_rate<ND, CART, TW>(g, q, w);
-    if (r > best) best = r;
+    best = raise_to(best, r);
   }
   cfl_block_max<TW>(best, mx);
 }

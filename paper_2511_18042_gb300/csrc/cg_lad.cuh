@@ -39,9 +39,9 @@ __device__ __forceinline__ void lad_fields(const DevGrid& g, const T* w, T* f) {
   T rho = w[0], p = w[IP];
 #pragma unroll
   for (int k = 0; k < ND; ++k) f[k] = w[1 + k];
-  f[ND] = gconst<T>(g.gm2, g.f_gm2) * p / rho;
+  f[ND] = div_t(gconst<T>(g.gm2, g.f_gm2) * p, rho);
   f[ND + 1] = rho;
-  f[ND + 2] = p / (rho * gconst<T>(g.gm1, g.f_gm1));
+  f[ND + 2] = div_t(p, rho * gconst<T>(g.gm1, g.f_gm1));
 }
 
 __device__ __forceinline__ void box_coords(const Box& b, long long e, int* c) {
@@ -237,7 +237,7 @@ __device__ __forceinline__ void k_lad_coef_body(const VBlock& vb, const DevGrid&
     T rho = w[0], p = w[IP];
     long long fq = fbx.at(c[0], c[1], c[2]);
     T Tt = fb[ND * fs + fq];
-    T cs = sqrt(gconst<T>(g.gamma, g.f_gamma) * p / rho);
+    T cs = sqrt_t(div_t(gconst<T>(g.gamma, g.f_gamma) * p, rho));
     T div = dv[e0];
     T curl2 = T(0);
     auto G = [&](int f, int m) { return gr[(f * ND + m) * bs + e0]; };
@@ -254,7 +254,7 @@ __device__ __forceinline__ void k_lad_coef_body(const VBlock& vb, const DevGrid&
     // pipe) are formed only where div < 0, each as in the full product.
     const bool comp = div < T(0);
     T fsw = T(0), gmr = T(0), gme;
-    if (comp) fsw = (div * div) / (div * div + curl2 + T(1e-32));
+    if (comp) fsw = div_t(div * div, div * div + curl2 + T(1e-32));
     if constexpr (sizeof(T) == 4) {
       // |grad rho| and |grad e| without squaring: in FP32 a square under
       // ~1e-38 flushes, and |x . grad| / (0 + 1e-32) would then inflate the
@@ -265,12 +265,12 @@ __device__ __forceinline__ void k_lad_coef_body(const VBlock& vb, const DevGrid&
       gme = G(ND + 2, 0) * G(ND + 2, 0);
 #pragma unroll
       for (int m = 1; m < ND; ++m) gme = gme + G(ND + 2, m) * G(ND + 2, m);
-      gme = sqrt(gme);
+      gme = sqrt_t(gme);
       if (comp) {
         gmr = G(ND + 1, 0) * G(ND + 1, 0);
 #pragma unroll
         for (int m = 1; m < ND; ++m) gmr = gmr + G(ND + 1, m) * G(ND + 1, m);
-        gmr = sqrt(gmr);
+        gmr = sqrt_t(gmr);
       }
     }
     T sb = T(0), sk = T(0);
@@ -279,7 +279,7 @@ __device__ __forceinline__ void k_lad_coef_body(const VBlock& vb, const DevGrid&
       long long st = l == 0 ? 1 : (l == 1 ? (long long)b3.ext[0] : (long long)b3.ext[0] * b3.ext[1]);
       long long fst = l == 0 ? 1 : (l == 1 ? (long long)fbx.ext[0] : (long long)fbx.ext[0] * fbx.ext[1]);
       const T* ev = fb + (ND + 2) * fs + fq;
-      T d4e = (ev[-2 * fst] + ev[2 * fst]) - T(4.0) * (ev[-fst] + ev[fst]) + T(6.0) * ev[0];
+      T d4e = add_scaled(ev[-2 * fst] + ev[2 * fst], T(-4.0), ev[-fst] + ev[fst]) + T(6.0) * ev[0];
       // projections x_l . grad of rho (pr) and e (pe), x_l = dx/dxi_l
       T pr = T(0), pe;
       if (CART) {
@@ -296,18 +296,18 @@ __device__ __forceinline__ void k_lad_coef_body(const VBlock& vb, const DevGrid&
           for (int m = 1; m < ND; ++m) pr = pr + to_t<T>(g.dxl[(l * ND + m) * g.NP + pq]) * G(ND + 1, m);
         }
       }
-      T Dk = fabs(pe) / (gme + T(1e-32));
+      T Dk = div_t(fabs(pe), gme + T(1e-32));
       T tk = d4e * Dk;
       sk = (l == 0) ? tk : sk + tk;
       if (comp) {
-        T d4d = (dv[e0 - 2 * st] + dv[e0 + 2 * st]) - T(4.0) * (dv[e0 - st] + dv[e0 + st]) + T(6.0) * div;
-        T Db = fabs(pr) / (gmr + T(1e-32));
+        T d4d = add_scaled(dv[e0 - 2 * st] + dv[e0 + 2 * st], T(-4.0), dv[e0 - st] + dv[e0 + st]) + T(6.0) * div;
+        T Db = div_t(fabs(pr), gmr + T(1e-32));
         T tb = d4d * Db * Db;
         sb = (l == 0) ? tb : sb + tb;
       }
     }
     bt[q] = c_beta * rho * fsw * fabs(sb);
-    kp[q] = c_kappa * (rho * cs / Tt) * fabs(sk);
+    kp[q] = c_kappa * div_t(rho * cs, Tt) * fabs(sk);
   }
 }
 
@@ -400,7 +400,7 @@ __device__ __forceinline__ void nodeflux_at(const DevGrid& g, int l, const T* __
       q2 = w[1] * w[1];
 #pragma unroll
       for (int m = 1; m < ND; ++m) q2 = q2 + w[1 + m] * w[1 + m];
-      T E = p / gconst<T>(g.gm1, g.f_gm1) + T(0.5) * rho * q2;
+      T E = add_scaled(div_t(p, gconst<T>(g.gm1, g.f_gm1)), T(0.5), rho * q2);
       fc[0] = rho * U;
 #pragma unroll
       for (int m = 0; m < ND; ++m) fc[1 + m] = (CART && m != l) ? rho * w[1 + m] * U : rho * w[1 + m] * U + xi[m] * p;
@@ -553,10 +553,10 @@ __device__ __forceinline__ void k_lad_viscoef_body(const VBlock& vb, const DevGr
     load_state<ND, false, T, T>(g, W, c[0], c[1], c[2], w);
     T rho = w[0], p = w[IP];
     long long sq = scalar_src(g, c[0], c[1], c[2]);
-    T Tt = T(g.gm2) * p / rho;
+    T Tt = div_t(T(g.gm2) * p, rho);
     T S = T(g.suth);
-    T mu = Tt * sqrt(Tt) * (T(1.0) + S) / (Tt + S) / T(g.re);
-    T kth = mu / T(g.kc);
+    T mu = div_t(div_t(Tt * sqrt_t(Tt) * (T(1.0) + S), Tt + S), T(g.re));
+    T kth = div_t(mu, T(g.kc));
     T lam = (ART ? bt[sq] : T(0)) - T(2.0 / 3.0) * mu;
     T kap = (ART ? kp[sq] : T(0)) + kth;
     vco[e] = mu;
