@@ -690,9 +690,14 @@ static GbrCfg gbr_cfg(const cg_solver* s) {
   q.f_thr = (float)q.thr;
   q.f_eps = (float)q.eps;
   q.f_alpha = (float)q.alpha;
-  const double big = 0x1p400;
-  q.f64_fast = q.gm1 > 1.0 / big && q.gm1 < big && q.gamma > 1.0 / big && q.gamma < big && q.eps >= 0.0 && q.eps < big &&
-               fabs(q.alpha) < big;
+  // gbr_flux_f64 takes the parameters and the constants of a Cartesian frame
+  // as operands in range
+  auto fits = [](double x) { return fabs(x) > 0x1p-100 && fabs(x) < 0x1p100; };
+  q.f64_fast = fits(q.gm1) && q.gm1 > 0.0 && fits(q.gamma) && q.gamma > 0.0 && q.eps >= 0.0 && q.eps < 1.0 &&
+               (q.alpha == 0.0 || fits(q.alpha));
+  if (!s->dg.curv)
+    for (int d = 0; d < s->nd; ++d)
+      q.f64_fast = q.f64_fast && fits(s->dg.cxh[d]) && fits(s->dg.cg2[d]) && fits(s->dg.cig2[d]);
   q.d_gm1 = host_divisor(q.f64_fast ? q.gm1 : 1.0);
   return q;
 }
@@ -922,6 +927,7 @@ static int gbr_sweeps(cg_solver* s, bool compact, StageArgs A, cudaStream_t st, 
     A.Gd = s->G[d];
     A.Gdf = reinterpret_cast<const float*>(s->G[d]);
     A.gdLB = s->gdLB[d];
+    A.compact = compact ? 1 : 0;
     A.iface_out = (s->iface_out && s->iface_dir == d) ? s->iface_out : nullptr;
     int rc;
     if (s->dg.curv) rc = compact ? sweep_dir<ND, false, true>(s, d, A, st) : sweep_dir<ND, false, false>(s, d, A, st);

@@ -391,7 +391,16 @@ template <typename T = double>
 __device__ __forceinline__ T d6(T m3, T m2, T m1, T p1, T p2, T p3) {
   return T(0.75) * (p1 - m1) - T(3.0 / 20.0) * (p2 - m2) + T(1.0 / 60.0) * (p3 - m3);
 }
+// (products by P; the FP64 forms round as the plain ones)
+template <typename T, class PR>
+__device__ __forceinline__ T d6(const PR& P, T m3, T m2, T m1, T p1, T p2, T p3) {
+  return P.kz(T(0.75), p1 - m1) - P.kz(T(3.0 / 20.0), p2 - m2) + P.kz(T(1.0 / 60.0), p3 - m3);
+}
 // explicit fourth-order central first derivative (E4)
+template <typename T, class PR>
+__device__ __forceinline__ T d4(const PR& P, T m2, T m1, T p1, T p2) {
+  return P.kz(T(2.0 / 3.0), p1 - m1) - P.kz(T(1.0 / 12.0), p2 - m2);
+}
 template <typename T = double>
 __device__ __forceinline__ T d4(T m2, T m1, T p1, T p2) {
   return T(2.0 / 3.0) * (p1 - m1) - T(1.0 / 12.0) * (p2 - m2);

@@ -192,6 +192,98 @@ inline Divisor host_divisor(double x) {
   return D;
 }
 
+// ---------------------------------------------------------------- products
+// A correctly rounded product on the integer pipes: the 106-bit product of the
+// significands in four 32 x 32 multiply-adds, normalised by at most one bit,
+// rounded to nearest even on the bits below.  About 30 integer instructions,
+// 18.9 clocks a warp on one SM where a DMUL is 18.7, but on other pipes: a
+// loop of one addition and one product takes 18.7 clocks instead of 37.3 (the
+// same probe).  So the products of an FP64-bound kernel are free as long as
+// they are no more than its additions.
+// a: in range; b: in range, or zero where ZB.
+__device__ __forceinline__ unsigned long long mad_wide(unsigned a, unsigned b, unsigned long long c) {
+  return (unsigned long long)a * b + c;
+}
+template <bool ZB>
+__device__ __forceinline__ double mul_int(double a, double b) {
+  const unsigned ah = (unsigned)__double2hiint(a), al = (unsigned)__double2loint(a);
+  const unsigned bh = (unsigned)__double2hiint(b), bl = (unsigned)__double2loint(b);
+  const unsigned a1 = __funnelshift_l(al, ah, 11) | 0x80000000u, a0 = al << 11;  // [2^63, 2^64)
+  const unsigned b1 = (bh & 0x000fffffu) | 0x00100000u;                         // [2^52, 2^53)
+  const unsigned long long t0 = mad_wide(a0, bl, 0ull), t1 = mad_wide(a1, bl, t0 >> 32),
+                           t2 = mad_wide(a0, b1, (unsigned)t1);
+  const unsigned long long H = mad_wide(a1, b1, t1 >> 32) + (t2 >> 32);  // [2^51, 2^53)
+  const unsigned h1 = hi_of(H), h0 = (unsigned)H, l1 = (unsigned)t2, l0 = (unsigned)t0;
+  const unsigned n = 1u - (h1 >> 20);
+  const unsigned m1 = __funnelshift_l(h0, h1, n), m0 = __funnelshift_l(l1, h0, n);
+  const unsigned low = l0 << n;
+  const unsigned f = __funnelshift_l(l0, l1, n) | (low < 1u ? low : 1u);
+  const unsigned long long M = u64_of(m1, m0) + (((unsigned long long)f + 0x7fffffffu + (m0 & 1u)) >> 32);
+  const unsigned rh = hi_of(M) + (ah & 0xfff00000u) + (bh & 0xfff00000u) - (1023u << 20) - (n << 20);
+  const bool zero = ZB && ((bh & 0x7fffffffu) | bl) == 0u;
+  return __hiloint2double((int)(zero ? (ah ^ bh) & 0x80000000u : rh), (int)(zero ? 0u : (unsigned)M));
+}
+
+// Products of an evaluation that collects its range tests.  The additions of
+// an evaluation hold the FP64 pipe anyway; a product with a factor that is
+// known to be in range (a constant, a density) goes to the integer pipes (kk,
+// kz), one of two unknown factors stays on the FP64 pipe (zz): testing two
+// operands costs as much as the product, and with every product on the
+// integer pipes the interface sweep is bound by its code size (instruction
+// fetch) instead: 1.94 and 1.89 ms of MEG6 sweeps against 1.92 and 1.85.
+struct F64Products {
+  F64Range& R;
+  static __device__ __forceinline__ double zz(double a, double b) { return a * b; }
+  // a in range, b any (zero, or tested here)
+  __device__ __forceinline__ double kz(double a, double b) const {
+    R.any0(b);
+    return mul_int<true>(a, b);
+  }
+  // both in range
+  static __device__ __forceinline__ double kk(double a, double b) { return mul_int<false>(a, b); }
+};
+struct PlainProducts {
+  template <typename T>
+  static __device__ __forceinline__ T zz(T a, T b) { return a * b; }
+  template <typename T>
+  static __device__ __forceinline__ T kz(T a, T b) { return a * b; }
+  template <typename T>
+  static __device__ __forceinline__ T kk(T a, T b) { return a * b; }
+};
+
+// A factor used as known to be in range: tested with the rest.
+__device__ __forceinline__ void require_range(const F64Products& P, double a) { P.R.any(a); }
+template <typename T>
+__device__ __forceinline__ void require_range(const PlainProducts&, T) {}
+
+// Keeps a rare branch a branch: an FP64 instruction that is predicated off holds
+// the pipe as long as one that runs (probe: a predicated DMUL beside a product
+// on the integer pipes, 36.4 clocks; behind a call, 18.7), and the compiler
+// predicates short branches that hold no call.
+static __device__ __noinline__ void rare_branch() { asm volatile(""); }
+
+// Where the additions are few beside the products and the loads, it takes less:
+// us a pass of the triple point 1792 x 768 with plain and with integer-pipe
+// products: Gaussian 431 and 276, interface LAD fluxes 334 and 216, E4 gradients
+// 503 and 289, sensor 462 and 333.
+//
+// f(P) with the products of an FP64 evaluation on the integer pipes, and again
+// with plain products where an operand was out of range (the same values
+// otherwise); float: plain products.
+template <typename T, class F>
+__device__ __forceinline__ void with_products(F f) {
+  if constexpr (sizeof(T) == 8) {
+    F64Range R;
+    f(F64Products{R});
+    if (!R.ok()) {
+      rare_branch();
+      f(PlainProducts{});
+    }
+  } else {
+    f(PlainProducts{});
+  }
+}
+
 // ---------------------------------------------------------------- comparisons
 // Comparisons of finite doubles on their bit patterns (a DSETP holds the FP64
 // pipe as long as an addition does).

@@ -2,6 +2,7 @@
 // limiting and the wave-appropriate selection of Eq. (8), HLLC flux of
 // Eq. (9)-(10), and the kernels of one RK stage.
 #pragma once
+#include <type_traits>
 #include "cg_device.cuh"
 
 namespace cgk {
@@ -248,11 +249,13 @@ __device__ __forceinline__ void gbr_flux(const GbrCfg& q, const DevGrid& g, cons
 //   * the characteristic variables of the outer stencil nodes only where MP5
 //     reads them (the acoustic and shear waves of a flagged interface, the
 //     entropy wave where Eq. (8) limits it);
+//   * products with a factor known to be in range on the integer pipes (IM);
 //   * on a Cartesian grid whose unit normals are exactly 1 (UN) no
 //     multiplication by them.
-// Measured (triple point 1792 x 768, MEG6): FP64 instructions an interface 569
-// -> 272 (with the staging and the epilogue), FP64 pipe 80 % busy; the sweep
-// 1.51 -> 0.79 ms a launch, the whole step 9.98 -> 5.60 ms.
+// Measured (triple point 1792 x 768, MEG6, with the staging and the epilogue):
+// FP64 instructions an interface 569 -> 272 without the products on the integer
+// pipes, about 190 with them; the sweep 1.51 -> 0.76 -> 0.63 ms a launch, the
+// whole step 9.98 -> 5.23 -> 4.26 ms.
 // Returns false where an operand is out of the range of these forms (a state
 // that is not positive, NaN, extreme magnitudes): the caller then repeats the
 // interface with gbr_flux.
@@ -298,12 +301,28 @@ static __device__ __noinline__ Mp5Pair mp5_pair_f64(double v0, double v1, double
   return o;
 }
 
+// sum_m a[m] u[m] over the structurally non-zero a[m], in index order (sdot)
+template <int ND, bool CART, int DIR, int VEC, class PR>
+__device__ __forceinline__ double sdot_f64(const PR& P, const double* a, const double* u) {
+  double s = 0.0;
+  bool first = true;
+#pragma unroll
+  for (int m = 0; m < ND; ++m) {
+    if (!frame_nz(CART, ND, DIR, VEC, m)) continue;
+    const double t = CART ? P.kz(a[m], u[m]) : P.zz(a[m], u[m]);
+    s = first ? t : s + t;
+    first = false;
+  }
+  return s;
+}
+
 // characteristic variables of a primitive vector (to_char's values)
-template <int ND, bool CART, int DIR, bool UN>
-__device__ __forceinline__ void to_char_f64(const Frame<ND, double>& f, const double* w, double* c) {
+template <int ND, bool CART, int DIR, bool UN, class PR>
+__device__ __forceinline__ void to_char_f64(const PR& P, const Frame<ND, double>& f, const double* w,
+                                            double* c) {
   constexpr int IP = ND + 1;
-  const double un = UN ? by_sign(f.n[DIR], w[1 + DIR]) : sdot<ND, CART, DIR, 0, double>(f.n, w + 1);
-  const double a = f.ha * w[IP], b = f.hb * un;
+  const double un = UN ? by_sign(f.n[DIR], w[1 + DIR]) : sdot_f64<ND, CART, DIR, 0>(P, f.n, w + 1);
+  const double a = P.kz(f.ha, w[IP]), b = P.kz(f.hb, un);
   c[0] = a - b;
   c[1] = __fma_rn(-2.0, a, w[0]);
   c[IP] = a + b;
@@ -312,84 +331,95 @@ __device__ __forceinline__ void to_char_f64(const Frame<ND, double>& f, const do
     if (UN && ND >= 2 && frame_nz(CART, ND, DIR, 1, m)) c[2] = by_sign(f.t1[m], w[1 + m]);
     if (UN && ND == 3 && frame_nz(CART, ND, DIR, 2, m)) c[3] = by_sign(f.t2[m], w[1 + m]);
   }
-  if (!UN && ND >= 2) c[2] = sdot<ND, CART, DIR, 1, double>(f.t1, w + 1);
-  if (!UN && ND == 3) c[3] = sdot<ND, CART, DIR, 2, double>(f.t2, w + 1);
+  if (!UN && ND >= 2) c[2] = sdot_f64<ND, CART, DIR, 1>(P, f.t1, w + 1);
+  if (!UN && ND == 3) c[3] = sdot_f64<ND, CART, DIR, 2>(P, f.t2, w + 1);
 }
 
-template <int ND, bool CART, int DIR, bool UN>
-__device__ __forceinline__ void from_char_f64(const Frame<ND, double>& f, double cb2, const double* c, double* w) {
+// from_char's values; cb2 = cb^2
+template <int ND, bool CART, int DIR, bool UN, class PR>
+__device__ __forceinline__ void from_char_f64(const PR& P, const Frame<ND, double>& f, double cb2,
+                                              const double* c, double* w) {
   constexpr int IP = ND + 1;
-  if (!UN) {
-    from_char<ND, CART, DIR, double>(f, c, w);
-    return;
-  }
   const double s = c[0] + c[IP];
+  const double un = P.kz(f.cr, c[IP] - c[0]);
   w[0] = c[1] + s;
-  w[IP] = cb2 * s;
+  w[IP] = P.kz(cb2, s);
 #pragma unroll
   for (int m = 0; m < ND; ++m) {
-    if (m == DIR) w[1 + m] = by_sign(f.n[m], (c[IP] - c[0]) * f.cr);
-    else if (ND >= 2 && frame_nz(CART, ND, DIR, 1, m)) w[1 + m] = by_sign(f.t1[m], c[2]);
-    else w[1 + m] = by_sign(f.t2[m], c[3]);
+    if (UN) {
+      if (m == DIR) w[1 + m] = by_sign(f.n[m], un);
+      else if (ND >= 2 && frame_nz(CART, ND, DIR, 1, m)) w[1 + m] = by_sign(f.t1[m], c[2]);
+      else w[1 + m] = by_sign(f.t2[m], c[3]);
+      continue;
+    }
+    auto t = [&](double a, double b) { return CART ? P.kz(a, b) : P.zz(a, b); };
+    double u = 0.0;
+    bool any = false;
+    if (frame_nz(CART, ND, DIR, 0, m)) { u = t(f.n[m], un); any = true; }
+    if (ND >= 2 && frame_nz(CART, ND, DIR, 1, m)) { u = any ? u + t(f.t1[m], c[2]) : t(f.t1[m], c[2]); any = true; }
+    if (ND == 3 && frame_nz(CART, ND, DIR, 2, m)) { u = any ? u + t(f.t2[m], c[3]) : t(f.t2[m], c[3]); any = true; }
+    w[1 + m] = u;
   }
 }
 
-template <int ND, bool CART, int DIR>
-__device__ __forceinline__ void hllc_f64(const GbrCfg& q, const double* WL, const double* WR, const double* xi,
+template <int ND, bool CART, int DIR, class PR>
+__device__ __forceinline__ void hllc_f64(const PR& P, const GbrCfg& q, const double* WL, const double* WR, const double* xi,
                                          double g2, double g, double ig2, double* F, F64Range& R) {
   constexpr int IP = ND + 1;
+  auto xm = [&](double a, double b) { return CART ? P.kz(a, b) : P.zz(a, b); };  // by a metric component
   const double rL = WL[0], pL = WL[IP], rR = WR[0], pR = WR[IP];
   R.pos(rL);
   R.pos(pL);
   R.pos(rR);
   R.pos(pR);
-  const double UL = sdot<ND, CART, DIR, 0, double>(xi, WL + 1);
-  const double UR = sdot<ND, CART, DIR, 0, double>(xi, WR + 1);
+  const double UL = sdot_f64<ND, CART, DIR, 0>(P, xi, WL + 1);
+  const double UR = sdot_f64<ND, CART, DIR, 0>(P, xi, WR + 1);
   double SL, SR, EL, ER;
   {
-    double qL = WL[1] * WL[1], qR = WR[1] * WR[1];
+    double qL = P.zz(WL[1], WL[1]), qR = P.zz(WR[1], WR[1]);
 #pragma unroll
     for (int m = 1; m < ND; ++m) {
-      qL = qL + WL[1 + m] * WL[1 + m];
-      qR = qR + WR[1 + m] * WR[1 + m];
+      qL = qL + P.zz(WL[1 + m], WL[1 + m]);
+      qR = qR + P.zz(WR[1 + m], WR[1 + m]);
     }
-    EL = __fma_rn(0.5, rL * qL, div_by(pL, q.d_gm1));
-    ER = __fma_rn(0.5, rR * qR, div_by(pR, q.d_gm1));
+    EL = __fma_rn(0.5, P.kz(rL, qL), div_by(pL, q.d_gm1));
+    ER = __fma_rn(0.5, P.kz(rR, qR), div_by(pR, q.d_gm1));
     double cL, cR, HL, HR;
     {
       const Divisor D = divisor(rL);
       const double HN = EL + pL;
       R.any0(HN);
-      cL = sqrt_ranged(div_by(q.gamma * pL, D));
+      cL = sqrt_ranged(div_by(P.kk(q.gamma, pL), D));
       HL = div_by(HN, D);
     }
     {
       const Divisor D = divisor(rR);
       const double HN = ER + pR;
       R.any0(HN);
-      cR = sqrt_ranged(div_by(q.gamma * pR, D));
+      cR = sqrt_ranged(div_by(P.kk(q.gamma, pR), D));
       HR = div_by(HN, D);
     }
     const double sL = sqrt_ranged(rL), sR = sqrt_ranged(rR);
     const double iden = rcp_by(divisor(sL + sR));
     double uh[3];
 #pragma unroll
-    for (int m = 0; m < ND; ++m) uh[m] = (sL * WL[1 + m] + sR * WR[1 + m]) * iden;
-    double qh = uh[0] * uh[0];
+    for (int m = 0; m < ND; ++m) uh[m] = P.kz(iden, P.kz(sL, WL[1 + m]) + P.kz(sR, WR[1 + m]));
+    double qh = P.zz(uh[0], uh[0]);
 #pragma unroll
-    for (int m = 1; m < ND; ++m) qh = qh + uh[m] * uh[m];
-    const double Uh = sdot<ND, CART, DIR, 0, double>(xi, uh);
-    const double Hh = (sL * HL + sR * HR) * iden;
-    const double c2 = q.gm1 * __fma_rn(-0.5, qh, Hh);
+    for (int m = 1; m < ND; ++m) qh = qh + P.zz(uh[m], uh[m]);
+    const double Uh = sdot_f64<ND, CART, DIR, 0>(P, xi, uh);
+    const double Hh = P.kz(iden, P.kz(sL, HL) + P.kz(sR, HR));
+    const double c2 = P.kz(q.gm1, __fma_rn(-0.5, qh, Hh));
     R.pos(c2);
-    const double chg = sqrt_ranged(c2) * g;
-    SL = min_f64(UL - cL * g, Uh - chg);
-    SR = max_f64(UR + cR * g, Uh + chg);
+    const double chg = P.kk(g, sqrt_ranged(c2));
+    SL = min_f64(UL - P.kk(g, cL), Uh - chg);
+    SR = max_f64(UR + P.kk(g, cR), Uh + chg);
   }
   double Ss;
   {
     const double eR = SR - UR, eL = SL - UL;
-    const double num = rR * UR * eR - rL * UL * eL + (pL - pR) * g2, den = rR * eR - rL * eL;
+    const double num = P.zz(P.kz(rR, UR), eR) - P.zz(P.kz(rL, UL), eL) + P.kz(g2, pL - pR),
+                 den = P.kz(rR, eR) - P.kz(rL, eL);
     R.any0(num);
     R.any(den);
     Ss = div_by(num, divisor(den));
@@ -401,36 +431,47 @@ __device__ __forceinline__ void hllc_f64(const GbrCfg& q, const double* WL, cons
   for (int m = 0; m < ND; ++m) W[m] = left ? WL[1 + m] : WR[1 + m];
   const double r = left ? rL : rR, p = left ? pL : pR, U = left ? UL : UR, E = left ? EL : ER, S = left ? SL : SR;
   double ru[ND];
-  F[0] = r * U;
+  F[0] = P.kz(r, U);
 #pragma unroll
   for (int m = 0; m < ND; ++m) {
-    ru[m] = r * W[m];
-    F[1 + m] = frame_nz(CART, ND, DIR, 0, m) ? ru[m] * U + xi[m] * p : ru[m] * U;
+    ru[m] = P.kz(r, W[m]);
+    F[1 + m] = P.zz(ru[m], U);
+    if (frame_nz(CART, ND, DIR, 0, m)) F[1 + m] = F[1 + m] + xm(xi[m], p);
   }
-  F[IP] = (E + p) * U;
+  F[IP] = P.zz(E + p, U);
   if (!star) return;
-  const double SU = S - U, rSU = r * SU, SS = S - Ss, d = Ss - U;
+  const double SU = S - U, rSU = P.kz(r, SU), SS = S - Ss, d = Ss - U;
   R.any(rSU);
   R.any(SS);
   R.any0(E);
   const double fac = div_by(rSU, divisor(SS));
-  F[0] = F[0] + S * (fac - r);
+  F[0] = F[0] + P.zz(S, fac - r);
 #pragma unroll
   for (int m = 0; m < ND; ++m) {
-    const double qs = frame_nz(CART, ND, DIR, 0, m) ? fac * (W[m] + xi[m] * d * ig2) : fac * W[m];
-    F[1 + m] = F[1 + m] + S * (qs - ru[m]);
+    const double qs =
+        P.zz(fac, frame_nz(CART, ND, DIR, 0, m) ? W[m] + P.kz(ig2, xm(xi[m], d)) : W[m]);
+    F[1 + m] = F[1 + m] + P.zz(S, qs - ru[m]);
   }
-  const double qe = fac * (div_by(E, divisor(r)) + d * (Ss * ig2 + div_by(p, divisor(rSU))));
-  F[IP] = F[IP] + S * (qe - E);
+  const double qe = P.zz(fac, div_by(E, divisor(r)) + P.zz(d, P.kz(ig2, Ss) + div_by(p, divisor(rSU))));
+  F[IP] = F[IP] + P.zz(S, qe - E);
 }
 
+template <class PR>
+__device__ __forceinline__ PR make_products(F64Range& R) {
+  if constexpr (std::is_same_v<PR, F64Products>) return F64Products{R};
+  else return PR{};
+}
+
+// IM: products on the integer pipes (a contracting unit fuses them instead).
 // W(j, w): the primitives of stencil node i-2+j (j = 0..5); Wd(j, w), Wh(j, w):
 // first derivatives and halved second derivatives of node i+j (j = 0, 1).
-template <int ND, bool CART, int DIR, bool UN, class FW, class FD, class FH>
+template <int ND, bool CART, int DIR, bool UN, bool IM, class FW, class FD, class FH>
 __device__ __forceinline__ bool gbr_flux_f64(const GbrCfg& q, const DevGrid& g, FW ldW, FD ldD, FH ldH, bool disc,
                                              const double* xi, double* F) {
   constexpr int NV = ND + 2, IP = ND + 1;
   F64Range R;
+  using PR = std::conditional_t<IM, F64Products, PlainProducts>;
+  const PR P = make_products<PR>(R);
   if (!q.f64_fast) R.see(~0u);
   Frame<ND, double> fr;
   double g2, gg, ig2, xl[3];
@@ -485,48 +526,52 @@ __device__ __forceinline__ bool gbr_flux_f64(const GbrCfg& q, const DevGrid& g, 
     R.pos(rs);
     R.pos(ps);
     const Divisor D = divisor(rs);
-    fr.cb = sqrt_ranged(div_by(q.gamma * ps, D));
+    fr.cb = sqrt_ranged(div_by(P.kk(q.gamma, ps), D));
     const double ic = rcp_by(divisor(fr.cb));
-    fr.ic2 = ic * ic;
+    fr.ic2 = P.kk(ic, ic);
     fr.ha = scale2<-1>(fr.ic2);
-    fr.hb = scale2<-2>(rs * ic);
+    fr.hb = scale2<-2>(P.kk(rs, ic));
     fr.cr = scale2<1>(div_by(fr.cb, D));
-    cb2 = fr.cb * fr.cb;
+    cb2 = P.kk(fr.cb, fr.cb);
+    R.any(fr.ha);
+    R.any(fr.hb);
+    R.any(fr.cr);
+    R.any(cb2);
   }
   double CL[NV], CR[NV], C2[NV], C3[NV];
-  to_char_f64<ND, CART, DIR, UN>(fr, w2, C2);
-  to_char_f64<ND, CART, DIR, UN>(fr, w3, C3);
+  to_char_f64<ND, CART, DIR, UN>(P, fr, w2, C2);
+  to_char_f64<ND, CART, DIR, UN>(P, fr, w3, C3);
   const double c6 = 2.0 * (1.0 / 12.0);
   {
     double w[NV], c[NV];
     ldD(0, w);
-    to_char_f64<ND, CART, DIR, UN>(fr, w, c);
+    to_char_f64<ND, CART, DIR, UN>(P, fr, w, c);
 #pragma unroll
     for (int b = 0; b < NV; ++b) CL[b] = __fma_rn(0.5, c[b], C2[b]);
     ldH(0, w);
-    to_char_f64<ND, CART, DIR, UN>(fr, w, c);
+    to_char_f64<ND, CART, DIR, UN>(P, fr, w, c);
 #pragma unroll
-    for (int b = 0; b < NV; ++b) CL[b] = CL[b] + c[b] * c6;
+    for (int b = 0; b < NV; ++b) CL[b] = CL[b] + P.kz(c6, c[b]);
     ldD(1, w);
-    to_char_f64<ND, CART, DIR, UN>(fr, w, c);
+    to_char_f64<ND, CART, DIR, UN>(P, fr, w, c);
 #pragma unroll
     for (int b = 0; b < NV; ++b) CR[b] = __fma_rn(-0.5, c[b], C3[b]);
     ldH(1, w);
-    to_char_f64<ND, CART, DIR, UN>(fr, w, c);
+    to_char_f64<ND, CART, DIR, UN>(P, fr, w, c);
 #pragma unroll
-    for (int b = 0; b < NV; ++b) CR[b] = CR[b] + c[b] * c6;
+    for (int b = 0; b < NV; ++b) CR[b] = CR[b] + P.kz(c6, c[b]);
   }
   {  // entropy wave: MP criterion
     auto entropy = [&](int j) {
       double w[NV];
       ldW(j, w);
-      return __fma_rn(-2.0, fr.ha * w[IP], w[0]);
+      return __fma_rn(-2.0, P.kz(fr.ha, w[IP]), w[0]);
     };
     const double v1 = entropy(1), v2 = C2[1], v3 = C3[1], v4 = entropy(4);
     const double cl = CL[1], cr = CR[1], cc = 0.5 * (cl + cr), dv = v3 - v2;
-    const double umpL = v2 + minmod_f64(dv, q.alpha * (v2 - v1));
-    const double umpR = v3 + minmod_f64(-dv, q.alpha * (v3 - v4));
-    const double tL = (cl - v2) * (cl - umpL), tR = (cr - v3) * (cr - umpR);
+    const double umpL = v2 + minmod_f64(dv, P.zz(q.alpha, v2 - v1));
+    const double umpR = v3 + minmod_f64(-dv, P.zz(q.alpha, v3 - v4));
+    const double tL = P.zz(cl - v2, cl - umpL), tR = P.zz(cr - v3, cr - umpR);
     // finite and above eps
     const bool limL = bits64(tL) > bits64(q.eps) && __double2hiint(tL) < 0x7ff00000;
     const bool limR = bits64(tR) > bits64(q.eps) && __double2hiint(tR) < 0x7ff00000;
@@ -549,13 +594,13 @@ __device__ __forceinline__ bool gbr_flux_f64(const GbrCfg& q, const DevGrid& g, 
   } else {
     double C0[NV], C1[NV], C4[NV], C5[NV], w[NV];
     ldW(0, w);
-    to_char_f64<ND, CART, DIR, UN>(fr, w, C0);
+    to_char_f64<ND, CART, DIR, UN>(P, fr, w, C0);
     ldW(1, w);
-    to_char_f64<ND, CART, DIR, UN>(fr, w, C1);
+    to_char_f64<ND, CART, DIR, UN>(P, fr, w, C1);
     ldW(4, w);
-    to_char_f64<ND, CART, DIR, UN>(fr, w, C4);
+    to_char_f64<ND, CART, DIR, UN>(P, fr, w, C4);
     ldW(5, w);
-    to_char_f64<ND, CART, DIR, UN>(fr, w, C5);
+    to_char_f64<ND, CART, DIR, UN>(P, fr, w, C5);
 #pragma unroll
     for (int b = 0; b < NV; ++b) {
       if (b == 1) continue;
@@ -566,9 +611,9 @@ __device__ __forceinline__ bool gbr_flux_f64(const GbrCfg& q, const DevGrid& g, 
     }
   }
   double WL[NV], WR[NV];
-  from_char_f64<ND, CART, DIR, UN>(fr, cb2, CL, WL);
-  from_char_f64<ND, CART, DIR, UN>(fr, cb2, CR, WR);
-  hllc_f64<ND, CART, DIR>(q, WL, WR, xl, g2, gg, ig2, F, R);
+  from_char_f64<ND, CART, DIR, UN>(P, fr, cb2, CL, WL);
+  from_char_f64<ND, CART, DIR, UN>(P, fr, cb2, CR, WR);
+  hllc_f64<ND, CART, DIR>(P, q, WL, WR, xl, g2, gg, ig2, F, R);
   return R.ok();
 }
 

@@ -46,6 +46,7 @@ struct StageArgs {
   double* iface_out;          // diagnostics: interface fluxes [v][line][n+1] (NULL: none)
   const float* Wf;            // mixed form: the primitives stored in FP32
   const float* Gdf;           // mixed form: the compact gradients in FP32
+  int compact;                // FP64 sweep: take the gradients from Gd (the FP32 sweep is compiled for either)
 };
 
 // ---------------------------------------------------------------- stage epilogue
@@ -93,55 +94,72 @@ __device__ __forceinline__ void stage_epilogue(const DevGrid& g, const StageArgs
     if constexpr (MIX) return f2d_int(t);
     else return double(t);
   };
+  // FP64 form: the residuals r = -(J tot) and what multiplies them
+  using S = typename std::conditional<MIX, float, double>::type;  // plain products in the mixed form
   if (!A.rk) {
+    with_products<S>([&](auto P) {
+      if constexpr (!MIX) require_range(P, J);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) A.R[v * g.N + qi] = -(J * wide(tot[v]));
+      for (int v = 0; v < NV; ++v) out[v] = -P.kz(J, wide(tot[v]));
+    });
+#pragma unroll
+    for (int v = 0; v < NV; ++v) A.R[v * g.N + qi] = out[v];
     return;
   }
   const double dt = *A.dt;
-  if (A.stage == 1) {
-    [[maybe_unused]] float cJf = 0.f;
-    if constexpr (MIX) cJf = -(d2f_int(dt) * d2f_int(J));
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const double un = A.Un[v * g.N + qi];
-      if constexpr (MIX) {
-        out[v] = un + f2d_int(cJf * tot[v]);
-      } else {
-        const double r = -(J * wide(tot[v]));
-        out[v] = un + dt * r;
-      }
-      A.Uout[v * g.N + qi] = out[v];
-    }
-    return;
-  }
   [[maybe_unused]] float cJf = 0.f;
-  if constexpr (MIX) cJf = -((A.stage == 2 ? 0.25f : (2.0f / 3.0f)) * d2f_int(dt)) * d2f_int(J);
-  if (A.stage == 2) {
+  if constexpr (MIX) cJf = -((A.stage == 1 ? 1.0f : (A.stage == 2 ? 0.25f : (2.0f / 3.0f))) * d2f_int(dt)) * d2f_int(J);
+  double un[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const double un = A.Un[v * g.N + qi], uc = A.Uc[v * g.N + qi];
-      if constexpr (MIX) {
-        out[v] = __fma_rn(0.75, un, __fma_rn(0.25, uc, f2d_int(cJf * tot[v])));
-      } else {
-        const double r = -(J * wide(tot[v]));
-        out[v] = add_scaled(0.75 * un, 0.25, uc + dt * r);  // the product with 1/4 is exact
-      }
-      A.Uout[v * g.N + qi] = out[v];
-    }
-    return;
-  }
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const double un = A.Un[v * g.N + qi], uc = A.Uc[v * g.N + qi];
+  for (int v = 0; v < NV; ++v) un[v] = A.Un[v * g.N + qi];
+  if (A.stage == 1) {
     if constexpr (MIX) {
-      out[v] = __fma_rn(1.0 / 3.0, un, __fma_rn(2.0 / 3.0, uc, f2d_int(cJf * tot[v])));
+#pragma unroll
+      for (int v = 0; v < NV; ++v) out[v] = un[v] + f2d_int(cJf * tot[v]);
     } else {
-      const double r = -(J * wide(tot[v]));
-      out[v] = (1.0 / 3.0) * un + (2.0 / 3.0) * (uc + dt * r);
+      with_products<double>([&](auto P) {
+        require_range(P, J);
+        require_range(P, dt);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) out[v] = un[v] - P.kz(dt, P.kz(J, tot[v]));
+      });
     }
-    A.Uout[v * g.N + qi] = out[v];
+  } else {
+    double uc[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) uc[v] = A.Uc[v * g.N + qi];
+    if (A.stage == 2) {
+      if constexpr (MIX) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) out[v] = __fma_rn(0.75, un[v], __fma_rn(0.25, uc[v], f2d_int(cJf * tot[v])));
+      } else {
+        with_products<double>([&](auto P) {
+          require_range(P, J);
+          require_range(P, dt);
+#pragma unroll
+          for (int v = 0; v < NV; ++v)  // the product with 1/4 is exact
+            out[v] = add_scaled(P.kz(0.75, un[v]), 0.25, uc[v] - P.kz(dt, P.kz(J, tot[v])));
+        });
+      }
+    } else {
+      if constexpr (MIX) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+          out[v] = __fma_rn(1.0 / 3.0, un[v], __fma_rn(2.0 / 3.0, uc[v], f2d_int(cJf * tot[v])));
+      } else {
+        with_products<double>([&](auto P) {
+          require_range(P, J);
+          require_range(P, dt);
+#pragma unroll
+          for (int v = 0; v < NV; ++v)
+            out[v] = P.kz(1.0 / 3.0, un[v]) + P.kz(2.0 / 3.0, uc[v] - P.kz(dt, P.kz(J, tot[v])));
+        });
+      }
+    }
   }
+#pragma unroll
+  for (int v = 0; v < NV; ++v) A.Uout[v * g.N + qi] = out[v];
+  if (A.stage != 3) return;
   bool bad;
   if constexpr (MIX) {
     bad = mixed_nonphysical<ND>(out);
@@ -251,13 +269,15 @@ __device__ __forceinline__ T sensor_zeta(const T (&gu)[3][3]) {
 
 // Physical velocity gradients gu[k][m] = sum_l (J xi_hat[l][m]) du[l][k] from
 // the index-space ones du[l][k] = d u_k / d xi_l at node c.
-template <int ND, bool CART, typename T>
-__device__ __forceinline__ void sensor_gu(const DevGrid& g, const int* c, const T (&du)[3][3], T (&gu)[3][3]) {
+template <int ND, bool CART, typename T, class PR>
+__device__ __forceinline__ void sensor_gu(const PR& P, const DevGrid& g, const int* c, const T (&du)[3][3], T (&gu)[3][3]) {
   if (CART) {
+#pragma unroll
+    for (int m = 0; m < ND; ++m) require_range(P, gconst<T>(g.cjxh[m], g.f_cjxh[m]));
 #pragma unroll
     for (int k = 0; k < ND; ++k)
 #pragma unroll
-      for (int m = 0; m < ND; ++m) gu[k][m] = gconst<T>(g.cjxh[m], g.f_cjxh[m]) * du[m][k];
+      for (int m = 0; m < ND; ++m) gu[k][m] = P.kz(gconst<T>(g.cjxh[m], g.f_cjxh[m]), du[m][k]);
   } else {
     long long pq = plin(g, c[0], c[1], c[2]);
     // J xi_hat: in the mixed form each factor is rounded to FP32 (on the
@@ -368,7 +388,7 @@ __device__ __forceinline__ void k_omega_body(const VBlock& vb, const DevGrid& g,
     }
     }
     T gu[3][3];
-    sensor_gu<ND, CART, T>(g, c, du, gu);
+    sensor_gu<ND, CART, T>(PlainProducts{}, g, c, du, gu);
     om[ob.at(c[0], c[1], c[2])] = phi * sensor_zeta<ND, T>(gu);
   }
 }
@@ -423,25 +443,10 @@ __global__ void __launch_bounds__(OMT_X * OMT_Y) k_omega_tile(DevGrid g, const T
   const int tx = threadIdx.x + OMT_H, ty = threadIdx.y + OMT_H;
   const T p0 = sP[ty][tx];
   T phi = T(0);
-  T du[3][3];
-  {  // x
-    const T pm = sP[ty][tx - 1], pp = sP[ty][tx + 1];
-    phi = raise_to(phi, sensor_phi<T>(pm, p0, pp));
-#pragma unroll
-    for (int k = 0; k < ND; ++k)
-      du[0][k] = d6<T>(sU[k][ty][tx - 3], sU[k][ty][tx - 2], sU[k][ty][tx - 1], sU[k][ty][tx + 1], sU[k][ty][tx + 2],
-                       sU[k][ty][tx + 3]);
-  }
-  {  // y
-    const T pm = sP[ty - 1][tx], pp = sP[ty + 1][tx];
-    phi = raise_to(phi, sensor_phi<T>(pm, p0, pp));
-#pragma unroll
-    for (int k = 0; k < ND; ++k)
-      du[1][k] = d6<T>(sU[k][ty - 3][tx], sU[k][ty - 2][tx], sU[k][ty - 1][tx], sU[k][ty + 1][tx], sU[k][ty + 2][tx],
-                       sU[k][ty + 3][tx]);
-  }
-  if constexpr (ND == 3) {  // z: direct loads in the interior, the boundary mapping elsewhere
-    T s[6][NV];
+  phi = raise_to(phi, sensor_phi<T>(sP[ty][tx - 1], p0, sP[ty][tx + 1]));
+  phi = raise_to(phi, sensor_phi<T>(sP[ty - 1][tx], p0, sP[ty + 1][tx]));
+  T s[ND == 3 ? 6 : 1][NV];  // z neighbours: direct loads in the interior, the boundary mapping elsewhere
+  if constexpr (ND == 3) {
     const bool inner = c[0] >= 0 && c[0] < g.n[0] && c[1] >= 0 && c[1] < g.n[1] && c[2] >= 3 && c[2] < g.n[2] - 3;
     if (inner) {
       const long long q = lin(g, c[0], c[1], c[2]), st = (long long)g.n[0] * g.n[1];
@@ -455,14 +460,22 @@ __global__ void __launch_bounds__(OMT_X * OMT_Y) k_omega_tile(DevGrid g, const T
 #pragma unroll 1
       for (int t = 0; t < 6; ++t) load_state<ND, false, T, T>(g, W, c[0], c[1], c[2] + (t < 3 ? t - 3 : t - 2), s[t]);
     }
-    const T pm = s[2][IP], pp = s[3][IP];
-    phi = raise_to(phi, sensor_phi<T>(pm, p0, pp));
-#pragma unroll
-    for (int k = 0; k < ND; ++k)
-      du[2][k] = d6<T>(s[0][1 + k], s[1][1 + k], s[2][1 + k], s[3][1 + k], s[4][1 + k], s[5][1 + k]);
+    phi = raise_to(phi, sensor_phi<T>(s[2][IP], p0, s[3][IP]));
   }
   T gu[3][3];
-  sensor_gu<ND, CART, T>(g, c, du, gu);
+  with_products<T>([&](auto P) {
+    T du[3][3];
+#pragma unroll
+    for (int k = 0; k < ND; ++k) {
+      du[0][k] = d6(P, sU[k][ty][tx - 3], sU[k][ty][tx - 2], sU[k][ty][tx - 1], sU[k][ty][tx + 1], sU[k][ty][tx + 2],
+                    sU[k][ty][tx + 3]);
+      du[1][k] = d6(P, sU[k][ty - 3][tx], sU[k][ty - 2][tx], sU[k][ty - 1][tx], sU[k][ty + 1][tx], sU[k][ty + 2][tx],
+                    sU[k][ty + 3][tx]);
+      if constexpr (ND == 3)
+        du[2][k] = d6(P, s[0][1 + k], s[1][1 + k], s[2][1 + k], s[3][1 + k], s[4][1 + k], s[5][1 + k]);
+    }
+    sensor_gu<ND, CART, T>(P, g, c, du, gu);
+  });
   om[ob.at(c[0], c[1], c[2])] = phi * sensor_zeta<ND, T>(gu);
 }
 
@@ -490,6 +503,7 @@ using LineCoef = LineCoefT<double>;
 
 // ---------------------------------------------------------------- C-GBR sweep
 constexpr int SWEEP_TL = 64;
+constexpr int SWEEP_THREADS = 256;
 // lines per tile: the default, and the candidates an autotuner may choose from
 // (LW * SWEEP_TL must be a multiple of the 256 threads of a block)
 __host__ __device__ constexpr int sweep_lw(int dir) { return dir == 0 ? 4 : 8; }
@@ -499,9 +513,12 @@ __host__ __device__ constexpr int sweep_smem_doubles() {
 }
 
 // Blocks per SM the register budget is sized for (256 threads a block):
-// * FP64: two (128 registers).  The 3D curvilinear sweep, with its frame and
-//   metric terms, spills about 300 bytes a thread there, to L1; at one block
-//   (8 warps an SM) it did not spill but ran 9-12 % slower on the 3D ramp.
+// * FP64, Cartesian: three (80 registers, up to 40 bytes a thread spill).  The
+//   products on the integer pipes make long dependent chains: the MEG6 sweeps
+//   of the triple point take 4.20 ms a step at two blocks, 3.77 at three and at
+//   four; blocks of 128 threads were slower (4.6: more distinct code in flight).
+// * FP64, curvilinear: two (128 registers): at three the 3D ramp's sweeps,
+//   which spill there, took 14.7 ms a step instead of 14.4.
 // * 1D/2D FP32: four (64 registers; up to 40 bytes a thread spill).  The
 //   kernel is latency-bound at two blocks, 16 warps an SM: four took the
 //   triple point's mixed MEG6 step from 1.24 to 1.02 ms.
@@ -509,15 +526,9 @@ __host__ __device__ constexpr int sweep_smem_doubles() {
 //   ramp 10-15 % faster than two.
 template <int ND, bool CART, typename T>
 __host__ __device__ constexpr int sweep_min_blocks() {
-  return sizeof(T) == 8 ? 2 : (ND <= 2 ? 4 : 3);
+  return sizeof(T) == 8 ? (CART ? 3 : 2) : (ND <= 2 ? 4 : 3);
 }
 
-// T = double: FP64 form; T = float: mixed form (FP32 reconstruction and
-// fluxes from FP64 primitives; FP64 flux differences, residual and RK update).
-// UNIT tags the translation unit that compiles the kernel (0: FP64 without
-// contraction, the oracle's operation order; 1: FP64 with fused multiply-add;
-// 2: FP32): the code is the same, the compilation flags differ, and distinct
-// instantiations keep the units' kernels apart.
 // The IEEE form of one interface flux of the FP64 sweep, from the staged tile:
 // the interfaces whose operands gbr_flux_f64 refuses.
 // io: the interface metrics in, the flux out.
@@ -545,9 +556,15 @@ static __device__ __noinline__ void gbr_flux_ieee(const GbrCfg& q, const DevGrid
   for (int v = 0; v < NV; ++v) io[v] = F[v];
 }
 
+// T = double: FP64 form; T = float: mixed form (FP32 reconstruction and
+// fluxes from FP64 primitives; FP64 flux differences, residual and RK update).
+// UNIT tags the translation unit that compiles the kernel (0: FP64 without
+// contraction, the oracle's operation order; 1: FP64 with fused multiply-add;
+// 2: FP32): the code is the same, the compilation flags differ, and distinct
+// instantiations keep the units' kernels apart.
 template <int ND, int DIR, bool CART, bool COMPACT, typename T, int LW, int UNIT, bool UN = false>
 __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid& g, const GbrCfg& q, const StageArgs& A) {
-  static_assert((SWEEP_TL * LW) % 256 == 0, "a tile must hold a multiple of the block's threads");
+  static_assert((SWEEP_TL * LW) % SWEEP_THREADS == 0, "a tile must hold a multiple of the block's threads");
   constexpr int NV = ND + 2;
   constexpr bool MIX = sizeof(T) == 4;
   constexpr int TL = SWEEP_TL;
@@ -658,7 +675,7 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
   if (A.mask) {
     int any = 0;
 #pragma unroll 1
-    for (int e = tid; e < TL * LW; e += blockDim.x) {
+    for (int e = tid; e < TL * LW; e += SWEEP_THREADS) {
       int a = DIR == 0 ? e % TL : e / LW;
       int l = DIR == 0 ? e / TL : e % LW;
       int i = i0 - 1 + a;
@@ -674,7 +691,7 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
   if (stage_tile) {
     // 1. primitives of the tile (ghosts resolved by the boundary conditions;
     // interior nodes read directly, the same values)
-    for (int e = tid; e < RW * LW; e += blockDim.x) {
+    for (int e = tid; e < RW * LW; e += SWEEP_THREADS) {
       int r = DIR == 0 ? e % RW : e / LW;
       int l = DIR == 0 ? e / RW : e % LW;
       int c[3] = {0, 0, 0};
@@ -696,7 +713,7 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
     }
     // sensor window: nodes above the threshold
     const T thr = gconst<T>(q.thr, q.f_thr);
-    for (int e = tid; e < RO * LW; e += blockDim.x) {
+    for (int e = tid; e < RO * LW; e += SWEEP_THREADS) {
       int r = DIR == 0 ? e % RO : e / LW;
       int l = DIR == 0 ? e / RO : e % LW;
       int x = i0 - 4 + r;
@@ -705,11 +722,11 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
     }
     __syncthreads();
     // 2. first derivatives along DIR on nodes i0-2 .. i0+TL
-    for (int e = tid; e < RD * LW; e += blockDim.x) {
+    for (int e = tid; e < RD * LW; e += SWEEP_THREADS) {
       int r = DIR == 0 ? e % RD : e / LW;
       int l = DIR == 0 ? e / RD : e % LW;
       T d[NV];
-      if (!COMPACT) {
+      if (MIX ? !COMPACT : !A.compact) {
         T m3[NV], m2[NV], m1[NV], p1[NV], p2[NV], p3[NV];
         ldn(sW, r, l, RW, m3);
         ldn(sW, r + 1, l, RW, m2);
@@ -717,8 +734,15 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
         ldn(sW, r + 4, l, RW, p1);
         ldn(sW, r + 5, l, RW, p2);
         ldn(sW, r + 6, l, RW, p3);
+        if constexpr (UNIT == 0) {
+          with_products<T>([&](auto P) {
 #pragma unroll
-        for (int v = 0; v < NV; ++v) d[v] = d6(m3[v], m2[v], m1[v], p1[v], p2[v], p3[v]);
+            for (int v = 0; v < NV; ++v) d[v] = d6(P, m3[v], m2[v], m1[v], p1[v], p2[v], p3[v]);
+          });
+        } else {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) d[v] = d6(m3[v], m2[v], m1[v], p1[v], p2[v], p3[v]);
+        }
       } else {
         int c[3] = {0, 0, 0};
         int x = i0 - 2 + r;
@@ -731,7 +755,7 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
     }
     __syncthreads();
     // 3. second derivatives on nodes i0-1 .. i0+TL-1
-    for (int e = tid; e < RDD * LW; e += blockDim.x) {
+    for (int e = tid; e < RDD * LW; e += SWEEP_THREADS) {
       int r = DIR == 0 ? e % RDD : e / LW;
       int l = DIR == 0 ? e / RDD : e % LW;
       T wm[NV], w0[NV], wp[NV], dm[NV], dp[NV], dd[NV];
@@ -750,10 +774,10 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
     __syncthreads();
   }
   // 4. interface fluxes i+1/2, i = i0-1+a
-  constexpr int PER = (TL * LW) / 256;
+  constexpr int PER = (TL * LW) / SWEEP_THREADS;
 #pragma unroll 1
   for (int k = 0; k < PER; ++k) {
-    int e = tid + k * 256;
+    int e = tid + k * SWEEP_THREADS;
     int a = DIR == 0 ? e % TL : e / LW;
     int l = DIR == 0 ? e / TL : e % LW;
     int i = i0 - 1 + a;
@@ -789,7 +813,7 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
         }
         gbr_flux<ND, CART, DIR, T>(q, g, Wst, Wd, Wdd, disc, xi, F);
       } else {
-        const bool good = gbr_flux_f64<ND, CART, DIR, UN>(
+        const bool good = gbr_flux_f64<ND, CART, DIR, UN, UNIT == 0>(
             q, g, [&](int j, double* w) { ldn(sW, a + 2 + j, l, RW, w); },
             [&](int j, double* w) { ldn(sD, a + 1 + j, l, RD, w); }, [&](int j, double* w) { ldn(sDD, a + j, l, RDD, w); },
             disc, xi, F);
@@ -821,7 +845,7 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
   }
   __syncthreads();
   // 5. flux differences of cells i0 .. i0+TL-2, residual and RK epilogue
-  for (int e = tid; e < (TL - 1) * LW; e += blockDim.x) {
+  for (int e = tid; e < (TL - 1) * LW; e += SWEEP_THREADS) {
     int a = DIR == 0 ? e % (TL - 1) : e / LW;
     int l = DIR == 0 ? e / (TL - 1) : e % LW;
     int c[3] = {0, 0, 0};
@@ -854,7 +878,7 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
 }
 
 template <int ND, int DIR, bool CART, bool COMPACT, typename T, int LW, int UNIT, bool UN>
-__global__ void __launch_bounds__(256, sweep_min_blocks<ND, CART, T>())
+__global__ void __launch_bounds__(SWEEP_THREADS, sweep_min_blocks<ND, CART, T>())
     k_gbr_sweep(const __grid_constant__ DevGrid g, const __grid_constant__ GbrCfg q, const __grid_constant__ StageArgs A) {
   k_gbr_sweep_body<ND, DIR, CART, COMPACT, T, LW, UNIT, UN>(hw_block(), g, q, A);
 }

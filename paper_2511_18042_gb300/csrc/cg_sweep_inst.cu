@@ -40,7 +40,7 @@ int launch_form(const DevGrid& g, const GbrCfg& q, const StageArgs& A, cudaStrea
     if (e != cudaSuccess) return (int)e;
     attr_set = true;
   }
-  k<<<sweep_grid<DIR, LW>(g), 256, smem, st>>>(g, q, A);
+  k<<<sweep_grid<DIR, LW>(g), SWEEP_THREADS, smem, st>>>(g, q, A);
   return (int)cudaGetLastError();
 }
 
@@ -48,7 +48,7 @@ int launch_form(const DevGrid& g, const GbrCfg& q, const StageArgs& A, cudaStrea
 // multiplications by it.
 template <int DIR, bool CART, bool COMPACT, int LW>
 int launch_one(const DevGrid& g, const GbrCfg& q, const StageArgs& A, cudaStream_t st) {
-  if constexpr (CART && sizeof(ST) == 8) {
+  if constexpr (CART && sizeof(ST) == 8 && SND <= 2) {
     if (g.unit[DIR]) return launch_form<DIR, CART, COMPACT, LW, true>(g, q, A, st);
   }
   return launch_form<DIR, CART, COMPACT, LW, false>(g, q, A, st);
@@ -56,8 +56,12 @@ int launch_one(const DevGrid& g, const GbrCfg& q, const StageArgs& A, cudaStream
 
 template <int DIR, int LW>
 int launch_kind(bool cart, bool compact, const DevGrid& g, const GbrCfg& q, const StageArgs& A, cudaStream_t st) {
-  if (cart) return compact ? launch_one<DIR, true, true, LW>(g, q, A, st) : launch_one<DIR, true, false, LW>(g, q, A, st);
-  return compact ? launch_one<DIR, false, true, LW>(g, q, A, st) : launch_one<DIR, false, false, LW>(g, q, A, st);
+  if constexpr (sizeof(ST) == 8) {  // one kernel for both kinds of gradients (StageArgs::compact)
+    return cart ? launch_one<DIR, true, false, LW>(g, q, A, st) : launch_one<DIR, false, false, LW>(g, q, A, st);
+  } else {
+    if (cart) return compact ? launch_one<DIR, true, true, LW>(g, q, A, st) : launch_one<DIR, true, false, LW>(g, q, A, st);
+    return compact ? launch_one<DIR, false, true, LW>(g, q, A, st) : launch_one<DIR, false, false, LW>(g, q, A, st);
+  }
 }
 
 template <int DIR>

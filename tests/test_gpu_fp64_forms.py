@@ -1,7 +1,7 @@
 """The FP64 forms of the interface sweep on the integer and FP32 pipes
 (csrc/cg_fp64.cuh) and the cases in which the sweep leaves them.
 
-Division, square root and the comparisons must equal the IEEE operations bit
+Division, square root, product and the comparisons must equal the IEEE operations bit
 for bit (they claim correct rounding, so there is no tolerance); the sweep must
 keep the parity of one RHS evaluation with the oracle (1e-13 of each
 variable's largest magnitude) where operands are out of the forms' range."""
@@ -33,6 +33,11 @@ __global__ void k(int op, const double* a, const double* b, double* x, double* y
     if (op == 3) { F64Range R; R.any0(u); x[i] = R.ok() ? div_by(u, host_divisor_sixty()) : u / 60.0; y[i] = u / 60.0; }
     if (op == 4) { x[i] = min_f64(u, v) + max_f64(u, v); y[i] = (u < v ? u : v) + (u > v ? u : v); }
     if (op == 5) { x[i] = minmod_f64(u, v); y[i] = (u > 0 && v > 0) ? (u < v ? u : v) : ((u < 0 && v < 0) ? (u > v ? u : v) : 0.0); }
+    if (op == 7) {
+      F64Range R; R.any(u);
+      const double p = F64Products{R}.kz(u, v);
+      x[i] = R.ok() ? p : u * v; y[i] = u * v;
+    }
     if (op == 6) { x[i] = nonneg(u) ? 1.0 : 0.0; y[i] = 0.0 <= u ? 1.0 : 0.0; }
   }
 }
@@ -78,7 +83,7 @@ def operands(seed, n=1 << 22):
     return x
 
 
-@pytest.mark.parametrize("op", range(7), ids=["div", "sqrt", "rcp", "sixty", "minmax", "minmod", "nonneg"])
+@pytest.mark.parametrize("op", range(8), ids=["div", "sqrt", "rcp", "sixty", "minmax", "minmod", "nonneg", "mul"])
 def test_forms_equal_ieee(forms, op):
     a, b = operands(op), operands(100 + op)
     rng = np.random.default_rng(200 + op)
