@@ -756,9 +756,7 @@ static bool rhs_in_solver(const LineJob<T>* jobs, int n) {
 
 template <typename T>
 static void launch_lines(const LineJob<T>* jobs, int n, cudaStream_t st) {
-  bool part = true;
-  for (int j = 0; j < n; ++j) part = part && jobs[j].L->pc.P >= 4;
-  if (part) {
+  if (lines_partitioned(jobs, n)) {
     PartJobsT<T> J;
     J.njobs = n;
     J.start[0] = 0;

@@ -232,8 +232,8 @@ __device__ __forceinline__ void thomas_column_c6(const LineCoefT<T>& lc, T* __re
 }
 
 // ---------------------------------------------------------------- partitioned solves
-// For few columns (a 1D grid, few lines) one thread per column leaves the GPU
-// idle: each column is split into P chunks of q rows solved concurrently.
+// For few columns (a 1D grid, few lines; at 1792 x 768 too) one thread per
+// column leaves the GPU idle: each column is split into P chunks of q rows solved concurrently.
 // Chunk k solves its own block T_k (local pivots), giving y = T_k^{-1} r and,
 // precomputed on the host, the responses V = T_k^{-1}(A_s e_s) and
 // W = T_k^{-1}(C_{e-1} e_{e-1}) to the unknowns just outside it, so that
@@ -242,6 +242,13 @@ __device__ __forceinline__ void thomas_column_c6(const LineCoefT<T>& lc, T* __re
 // solved by one thread per column; a last pass applies the correction (and,
 // for cyclic lines, the Sherman-Morrison term).  A block holds 32 columns
 // (lanes, coalesced) times the chunks.
+// In FP64 it is bound by the FP64 pipe and the three walks through the columns:
+// the LAD-C6 solves of the triple point 1792 x 768 took 2.60 ms a step with 10
+// FP64 instructions a row and rows past a batch predicated off; 1.38 with 7 (the
+// products on the integer pipes, the same values) and none predicated off.
+// Columns held in shared memory between the walks (8 or 4 columns a block, 3
+// blocks an SM) took 2.27 with the same arithmetic: too few warps for the serial
+// chains; in FP32 0.72 against 0.49.
 template <typename T>
 struct PartCoefT {
   const T* aL;   // sub-diagonal of row i inside its chunk (0 at chunk starts)
@@ -267,10 +274,20 @@ struct PartJobsT {
   int njobs;
 };
 
+// c x for a coefficient c known to be in range and any x, on the integer pipes
+__device__ __forceinline__ double coef_mul(double c, double x) {
+  F64Range R;
+  const double p = F64Products{R}.kz(c, x);
+  if (R.ok()) return p;
+  rare_branch();
+  return c * x;
+}
+
 // Partitioned forward elimination inside one chunk: y_i = (r_i - aL_i y_{i-1})
 // rd_i for i in [i0, i1), y_{i0-1} = 0 (aL is 0 at the chunk start), in place;
 // returns y_{i1-1}.  Batched like thomas_forward (the column values only: the
-// coefficients are shared by the block's columns and stay in cache).
+// coefficients are shared by the block's columns and stay in cache).  The FP32
+// form; FP64: part_forward_f64.
 template <typename T, int B>
 __device__ __forceinline__ T part_forward(T* __restrict__ col, long long nl, const T* __restrict__ aL,
                                           const T* __restrict__ rd, int i0, int i1) {
@@ -302,6 +319,108 @@ __device__ __forceinline__ T part_forward(T* __restrict__ col, long long nl, con
   for (int i = i0 + nfull * B; i < i1; ++i) {
     y = fma_t(-aL[i], y, col[(long long)i * nl]) * rd[i];
     col[(long long)i * nl] = y;
+  }
+  return y;
+}
+
+// The FP64 form of part_forward: the product with the reciprocal pivot on the
+// integer pipes (the same values).
+template <int B, typename T = double>
+__device__ __forceinline__ T part_forward_f64(T* __restrict__ col, long long nl, const PartCoefT<T>& pc, int i0, int i1) {
+  const int nfull = (i1 - i0) / B;
+  T y = T(0);
+  T v[B];
+  if (nfull > 0) {
+#pragma unroll
+    for (int k = 0; k < B; ++k) v[k] = col[(long long)(i0 + k) * nl];
+  }
+  for (int b = 0; b < nfull; ++b) {
+    const int base = i0 + b * B;
+    const bool more = b + 1 < nfull;
+    T nv[B];
+    if (more) {
+#pragma unroll
+      for (int k = 0; k < B; ++k) nv[k] = col[(long long)(base + B + k) * nl];
+    }
+#pragma unroll
+    for (int k = 0; k < B; ++k) {
+      y = coef_mul(pc.rd[base + k], fma_t(-pc.aL[base + k], y, v[k]));
+      col[(long long)(base + k) * nl] = y;
+    }
+    if (more) {
+#pragma unroll
+      for (int k = 0; k < B; ++k) v[k] = nv[k];
+    }
+  }
+#pragma unroll 1
+  for (int i = i0 + nfull * B; i < i1; ++i) {
+    y = coef_mul(pc.rd[i], fma_t(-pc.aL[i], y, col[(long long)i * nl]));
+    col[(long long)i * nl] = y;
+  }
+  return y;
+}
+
+// part_forward_f64 with the C6 right-hand sides formed on the way from the
+// source field (c6_forward; the same values): 4 FP64 instructions a row and
+// three products on the integer pipes instead of 7.  Full batches, then single rows: an FP64 instruction that is
+// predicated off holds the pipe all the same.
+template <int B, typename T = double>
+__device__ __forceinline__ T part_c6_forward_f64(T* __restrict__ col, long long nl, const PartCoefT<T>& pc, int i0, int i1,
+                                             const T* __restrict__ fp, long long st, int lo) {
+  const int p0 = pc.periodic ? i0 : lo + i0;
+  auto F = [&](int i) { return fp[(long long)(p0 + (i - i0)) * st]; };  // at row i's position
+  T y = T(0);
+  T w[B + 4];  // stencil values of rows i-2 .. i+B+1
+  w[0] = F(i0 - 2);
+  w[1] = F(i0 - 1);
+  w[2] = F(i0);
+  w[3] = F(i0 + 1);
+  int i = i0;
+  auto rhs = [&](int b) { return coef_mul(7.0 / 9.0, w[b + 3] - w[b + 1]) + coef_mul(1.0 / 36.0, w[b + 4] - w[b]); };
+  auto one = [&](T r) {  // row i with right-hand side r
+    y = coef_mul(pc.rd[i], fma_t(-pc.aL[i], y, r));
+    col[(long long)i * nl] = y;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) w[b] = w[b + 1];
+    ++i;
+  };
+  if (!pc.periodic && i0 == 0) {  // closure row
+    rare_branch();
+    w[4] = F(2);
+    one(d4(w[0], w[1], w[3], w[4]));
+  }
+  const int e1 = !pc.periodic && i1 == pc.m ? i1 - 1 : i1;
+  T nx[B];
+#pragma unroll
+  for (int b = 0; b < B; ++b) nx[b] = i + B <= e1 ? F(i + b + 2) : T(0);
+  for (; i + B <= e1; i += B) {
+    T t[B];
+#pragma unroll
+    for (int b = 0; b < B; ++b) w[b + 4] = nx[b];
+    if (i + 2 * B <= e1) {
+#pragma unroll
+      for (int b = 0; b < B; ++b) nx[b] = F(i + B + b + 2);
+    }
+#pragma unroll
+    for (int b = 0; b < B; ++b)
+      t[b] = rhs(b);
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      y = coef_mul(pc.rd[i + b], fma_t(-pc.aL[i + b], y, t[b]));
+      col[(long long)(i + b) * nl] = y;
+    }
+#pragma unroll
+    for (int b = 0; b < 4; ++b) w[b] = w[b + B];
+  }
+#pragma unroll 1
+  while (i < e1) {
+    w[4] = F(i + 2);
+    one(rhs(0));
+  }
+  if (i < i1) {  // closure row
+    rare_branch();
+    w[4] = F(i + 2);
+    one(d4(w[0], w[1], w[3], w[4]));
   }
   return y;
 }
@@ -353,28 +472,24 @@ __device__ __forceinline__ T c6_forward(T* __restrict__ col, long long nl, const
 
 // Partitioned update inside one chunk: x_i = y_i - V_i L_prev - W_i F_next
 // (- f z_i on a cyclic line) for i in [i0, i1), in place, B rows per batch.
-template <typename T, int B>
+template <typename T, int B, bool CYC>
 __device__ __forceinline__ void part_update(T* __restrict__ col, long long nl, const PartCoefT<T>& pc, int i0,
                                             int i1, T Lp, T Fn, T f) {
+  auto row = [&](int i, T v) {
+    T x = fma_t(-pc.V[i], Lp, v);
+    x = fma_t(-pc.W[i], Fn, x);
+    return CYC ? fma_t(-f, pc.z[i], x) : x;
+  };
   int i = i0;
   for (; i + B <= i1; i += B) {
     T v[B];
 #pragma unroll
     for (int k = 0; k < B; ++k) v[k] = col[(long long)(i + k) * nl];
 #pragma unroll
-    for (int k = 0; k < B; ++k) {
-      T x = fma_t(-pc.V[i + k], Lp, v[k]);
-      x = fma_t(-pc.W[i + k], Fn, x);
-      if (pc.periodic) x = fma_t(-f, pc.z[i + k], x);
-      col[(long long)(i + k) * nl] = x;
-    }
+    for (int k = 0; k < B; ++k) col[(long long)(i + k) * nl] = row(i + k, v[k]);
   }
-  for (; i < i1; ++i) {
-    T x = fma_t(-pc.V[i], Lp, col[(long long)i * nl]);
-    x = fma_t(-pc.W[i], Fn, x);
-    if (pc.periodic) x = fma_t(-f, pc.z[i], x);
-    col[(long long)i * nl] = x;
-  }
+#pragma unroll 1
+  for (; i < i1; ++i) col[(long long)i * nl] = row(i, col[(long long)i * nl]);
 }
 
 constexpr int kPartMax = 32;
@@ -383,6 +498,7 @@ template <typename T>
 __global__ void __launch_bounds__(1024) k_tri_part(PartJobsT<T> J) {
   __shared__ T sYF[kPartMax][32], sYL[kPartMax][32], sF[kPartMax][32], sL[kPartMax][32];
   __shared__ T sFact[32];
+  __shared__ T sCh[5 * kPartMax];  // the boundary recursion's factors: its serial loop would wait for each from memory
   // rows per batch: up to 1024 threads leave 64 registers a thread
   constexpr int PB = 4;
   const int lane = threadIdx.x, k = threadIdx.y;
@@ -394,6 +510,7 @@ __global__ void __launch_bounds__(1024) k_tri_part(PartJobsT<T> J) {
   const long long c = g0 - J.start[j] + lane;
   const bool active = c < nl * J.ncomp[j];
   T* col = J.x[j] + (active ? (c / nl) * pc.m * nl + c % nl : 0);
+  for (int i = k * 32 + lane; i < 5 * pc.P; i += 32 * blockDim.y) sCh[i] = pc.ch[i];
   const int s = k * pc.q, e = min(pc.m, s + pc.q);
   const bool mine = active && k < pc.P && s < e;
   if (mine) {
@@ -406,9 +523,11 @@ __global__ void __launch_bounds__(1024) k_tri_part(PartJobsT<T> J) {
       const int d = sr.lb.d;
       const long long st = d == 0 ? 1 : (d == 1 ? (long long)sr.fb.ext[0] : (long long)sr.fb.ext[0] * sr.fb.ext[1]);
       const T* fp = sr.f + (c / nl) * sr.fs + sr.fb.at(cc[0], cc[1], cc[2]);
-      y = c6_forward<T, PB>(col, nl, pc.aL, T(0), pc.rd, s, e, T(0), fp, st, sr.lb.lo, pc.m, pc.periodic != 0);
+      if constexpr (sizeof(T) == 8) y = part_c6_forward_f64<PB>(col, nl, pc, s, e, fp, st, sr.lb.lo);
+      else y = c6_forward<T, PB>(col, nl, pc.aL, T(0), pc.rd, s, e, T(0), fp, st, sr.lb.lo, pc.m, pc.periodic != 0);
     } else {
-      y = part_forward<T, PB>(col, nl, pc.aL, pc.rd, s, e);
+      if constexpr (sizeof(T) == 8) y = part_forward_f64<PB>(col, nl, pc, s, e);
+      else y = part_forward<T, PB>(col, nl, pc.aL, pc.rd, s, e);
     }
     sYL[k][lane] = y;
     y = thomas_backward<T, PB>(col, nl, pc.cp, s, e - 2, y);
@@ -419,7 +538,7 @@ __global__ void __launch_bounds__(1024) k_tri_part(PartJobsT<T> J) {
     // forward: F_k = pF_k + qF_k F_{k+1},  L_k = alpha_k + beta_k F_{k+1}
     T alpha = T(0), beta_prev = T(0);
     for (int kk = 0; kk < pc.P; ++kk) {
-      const T* h = pc.ch + 5 * kk;
+      const T* h = sCh + 5 * kk;
       T pF = fma_t(-h[3], alpha, sYF[kk][lane]) * h[0];
       alpha = fma_t(-h[4], fma_t(beta_prev, pF, alpha), sYL[kk][lane]);
       sF[kk][lane] = pF;
@@ -428,7 +547,7 @@ __global__ void __launch_bounds__(1024) k_tri_part(PartJobsT<T> J) {
     }
     T Fn = T(0);
     for (int kk = pc.P - 1; kk >= 0; --kk) {
-      const T* h = pc.ch + 5 * kk;
+      const T* h = sCh + 5 * kk;
       T F = fma_t(h[1], Fn, sF[kk][lane]);
       T L = fma_t(h[2], Fn, sL[kk][lane]);
       sF[kk][lane] = F;
@@ -441,8 +560,8 @@ __global__ void __launch_bounds__(1024) k_tri_part(PartJobsT<T> J) {
   if (mine) {
     const T Lp = k > 0 ? sL[k - 1][lane] : T(0);
     const T Fn = k + 1 < pc.P ? sF[k + 1][lane] : T(0);
-    const T f = pc.periodic ? sFact[lane] : T(0);
-    part_update<T, PB>(col, nl, pc, s, e, Lp, Fn, f);
+    if (pc.periodic) part_update<T, PB, true>(col, nl, pc, s, e, Lp, Fn, sFact[lane]);
+    else part_update<T, PB, false>(col, nl, pc, s, e, Lp, Fn, T(0));
   }
 }
 
