@@ -1301,7 +1301,6 @@ CG_API void cg_solver_destroy(cg_solver* s) {
     for (int side = 0; side < 2; ++side)
       if (s->prof[d][side]) cudaFree(s->prof[d][side]);
   if (s->mask) cudaFree(s->mask);
-  if (s->hyb_flag) cudaFree(s->hyb_flag);
   if (s->hyb_count) cudaFree(s->hyb_count);
   if (s->cflmax) cudaFree(s->cflmax);
   if (s->bad_flag) cudaFree(s->bad_flag);
@@ -1346,14 +1345,14 @@ CG_API int cg_solver_create(const cg_grid* g, const cg_params* p, cg_solver** ou
   if ((rc = dalloc(&s->W, NV)) || (rc = dalloc(&s->acc, NV)) || (rc = dalloc(&s->U1, NV)) ||
       (rc = dalloc(&s->U2, NV)) || (rc = dalloc(&s->om, (size_t)s->omBox.size())) || (rc = dalloc(&s->dt, 2)) ||
       (rc = dalloc(&s->t, 2)) || (rc = dalloc(&s->cflmax, 1)) || (rc = dalloc(&s->bad_flag, 1)) ||
-      (rc = dalloc(&s->bad_idx, 1)) || (rc = dalloc(&s->hyb_flag, 2)) || (rc = dalloc(&s->hyb_count, 1))) {
+      (rc = dalloc(&s->bad_idx, 1)) || (rc = dalloc(&s->hyb_count, 2))) {
     cg_solver_destroy(s);
     return rc;
   }
   cudaMemset(s->bad_flag, 0, sizeof(unsigned int));
   cudaMemset(s->bad_idx, 0xff, sizeof(unsigned long long));
-  cudaMemset(s->hyb_flag, 0, 2 * sizeof(int));
-  cudaMemset(s->hyb_count, 0, sizeof(unsigned long long));
+  cudaMemset(s->hyb_count, 0, 2 * sizeof(unsigned long long));
+  s->hyb_flag = reinterpret_cast<int*>(s->hyb_count + 1);  // cleared together, one memset a stage
   bool compact = p->scheme == CG_MIG4;
   long long mig4_cols = 0;
   for (int d = 0; d < s->nd; ++d) {

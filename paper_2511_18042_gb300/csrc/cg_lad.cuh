@@ -409,89 +409,104 @@ __device__ __forceinline__ void nodeflux_at(const DevGrid& g, int l, const T* __
 #pragma unroll
       for (int m = 0; m < ND; ++m) xi[m] = to_t<T>(g.xh[(l * ND + m) * g.NP + pq]);
     }
-    T rho = w[0], p = w[IP];
-    T fc[NV];
-    if (CONV) {
-      T U, q2;
-      if (CART) U = xi[l] * w[1 + l];
-      else {
-        U = xi[0] * w[1];
-#pragma unroll
-        for (int m = 1; m < ND; ++m) U = U + xi[m] * w[1 + m];
-      }
-      q2 = w[1] * w[1];
-#pragma unroll
-      for (int m = 1; m < ND; ++m) q2 = q2 + w[1 + m] * w[1 + m];
-      T E = add_scaled(div_t(p, gconst<T>(g.gm1, g.f_gm1)), T(0.5), rho * q2);
-      fc[0] = rho * U;
-#pragma unroll
-      for (int m = 0; m < ND; ++m) fc[1 + m] = (CART && m != l) ? rho * w[1 + m] * U : rho * w[1 + m] * U + xi[m] * p;
-      fc[IP] = (E + p) * U;
-    } else {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) fc[v] = T(0);
-    }
-    long long sq = scalar_src(g, c[0], c[1], c[2]);
-    long long be = b3.at(c[0], c[1], c[2]);
-    if (!PHYS) {
-      T tau = bt[sq] * dv[be];
-      T kap = kp[sq];
-      T fe = T(0);
-      bool first = true;
-#pragma unroll
-      for (int m = 0; m < ND; ++m) {
-        if (CART && m != l) continue;
-        T phi = w[1 + m] * tau + kap * gr[(ND * ND + m) * bs + be];
-        fe = first ? xi[m] * phi : fe + xi[m] * phi;
-        first = false;
-      }
-      F[0] = fc[0];
-#pragma unroll
-      for (int m = 0; m < ND; ++m) F[1 + m] = (CART && m != l) ? fc[1 + m] : fc[1 + m] - xi[m] * tau;
-      F[IP] = fc[IP] - fe;
-    } else {
+    const T rho = w[0], p = w[IP];
+    const long long be = b3.at(c[0], c[1], c[2]);
+    const T div = dv[be];
+    auto G = [&](int f, int m) { return gr[(f * ND + m) * bs + be]; };
+    [[maybe_unused]] T tau1, kap, mu, lam;
+    if constexpr (PHYS) {
       // mu, lambda = beta* - 2/3 mu and kappa* + mu / ((gamma-1) Pr M^2) of
       // the node, formed once per stage by k_lad_viscoef
       const long long vq = vbx.at(c[0], c[1], c[2]), vs = vbx.size();
-      T mu = vco[vq];
-      T lam = vco[vs + vq];
-      T kap = vco[2 * vs + vq];
-      T div = dv[be];
-      T tau[ND][ND];
+      mu = vco[vq];
+      lam = vco[vs + vq];
+      kap = vco[2 * vs + vq];
+    } else {
+      const long long sq = scalar_src(g, c[0], c[1], c[2]);
+      tau1 = bt[sq] * div;
+      kap = kp[sq];
+    }
+    T pg = T(0);  // p / (gamma - 1)
+    if (CONV) pg = div_t(p, gconst<T>(g.gm1, g.f_gm1));
+    with_products<T>([&](auto P) {
+      if (CART) require_range(P, xi[l]);
+      if (CONV) require_range(P, rho);
+      if (PHYS) {
+        require_range(P, mu);
+        require_range(P, kap);
+      }
+      auto X = [&](T a, T b) { return CART ? P.kz(a, b) : P.zz(a, b); };  // by a metric component
+      if (CONV) {
+        T U, q2;
+        if (CART) U = X(xi[l], w[1 + l]);
+        else {
+          U = X(xi[0], w[1]);
 #pragma unroll
-      for (int m = 0; m < ND; ++m)
-#pragma unroll
-        for (int a = 0; a < ND; ++a) {
-          T sm = gr[(a * ND + m) * bs + be] + gr[(m * ND + a) * bs + be];
-          tau[m][a] = mu * sm;
-          if (m == a) tau[m][a] = tau[m][a] + lam * div;
+          for (int m = 1; m < ND; ++m) U = U + X(xi[m], w[1 + m]);
         }
+        q2 = w[1] * w[1];
+#pragma unroll
+        for (int m = 1; m < ND; ++m) q2 = q2 + w[1 + m] * w[1 + m];
+        const T E = add_scaled(pg, T(0.5), P.kz(rho, q2));
+        F[0] = P.kz(rho, U);
+#pragma unroll
+        for (int m = 0; m < ND; ++m) {
+          F[1 + m] = P.kz(rho, w[1 + m]) * U;
+          if (!CART || m == l) F[1 + m] = F[1 + m] + X(xi[m], p);
+        }
+        F[IP] = (E + p) * U;
+      } else {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) F[v] = T(0);
+      }
       T fe = T(0);
       bool first = true;
+      if constexpr (!PHYS) {
 #pragma unroll
-      for (int m = 0; m < ND; ++m) {
-        if (CART && m != l) continue;
-        T phi = w[1] * tau[m][0];
-#pragma unroll
-        for (int a = 1; a < ND; ++a) phi = phi + w[1 + a] * tau[m][a];
-        phi = phi + kap * gr[(ND * ND + m) * bs + be];
-        fe = first ? xi[m] * phi : fe + xi[m] * phi;
-        first = false;
-      }
-      F[0] = fc[0];
-#pragma unroll
-      for (int a = 0; a < ND; ++a) {
-        T fv;
-        if (CART) fv = xi[l] * tau[l][a];
-        else {
-          fv = xi[0] * tau[0][a];
-#pragma unroll
-          for (int m = 1; m < ND; ++m) fv = fv + xi[m] * tau[m][a];
+        for (int m = 0; m < ND; ++m) {
+          if (CART && m != l) continue;
+          const T phi = w[1 + m] * tau1 + kap * G(ND, m);
+          fe = first ? X(xi[m], phi) : fe + X(xi[m], phi);
+          first = false;
         }
-        F[1 + a] = fc[1 + a] + (-fv);
+#pragma unroll
+        for (int m = 0; m < ND; ++m)
+          if (!CART || m == l) F[1 + m] = F[1 + m] - X(xi[m], tau1);
+        F[IP] = F[IP] - fe;
+      } else {
+        T tau[ND][ND];
+#pragma unroll
+        for (int m = 0; m < ND; ++m)
+#pragma unroll
+          for (int a = 0; a <= m; ++a) {  // symmetric: the sum of the two derivatives commutes
+            tau[m][a] = P.kz(mu, G(a, m) + G(m, a));
+            if (m == a) tau[m][a] = tau[m][a] + lam * div;
+            tau[a][m] = tau[m][a];
+          }
+#pragma unroll
+        for (int m = 0; m < ND; ++m) {
+          if (CART && m != l) continue;
+          T phi = w[1] * tau[m][0];
+#pragma unroll
+          for (int a = 1; a < ND; ++a) phi = phi + w[1 + a] * tau[m][a];
+          phi = phi + P.kz(kap, G(ND, m));
+          fe = first ? X(xi[m], phi) : fe + X(xi[m], phi);
+          first = false;
+        }
+#pragma unroll
+        for (int a = 0; a < ND; ++a) {
+          T fv;
+          if (CART) fv = X(xi[l], tau[l][a]);
+          else {
+            fv = X(xi[0], tau[0][a]);
+#pragma unroll
+            for (int m = 1; m < ND; ++m) fv = fv + X(xi[m], tau[m][a]);
+          }
+          F[1 + a] = F[1 + a] + (-fv);
+        }
+        F[IP] = F[IP] + (-fe);
       }
-      F[IP] = fc[IP] + (-fe);
-    }
+    });
   }
 }
 
@@ -522,8 +537,15 @@ __device__ __forceinline__ bool box_holds(const Box& b, const int* c) {
          c[2] + b.off[2] >= 0 && c[2] + b.off[2] < b.ext[2];
 }
 
+// Blocks an SM (of 128 threads): the 3D FP64 form would take 190 registers; held
+// to 128 the viscous node fluxes of the 3D ramp 256 x 96 x 64 take 1.58 ms a step
+// instead of 1.79 (1.86 with a launch for each direction).
+template <int ND, typename T>
+__host__ __device__ constexpr int nodeflux_blocks() {
+  return ND == 3 && sizeof(T) == 8 ? 4 : 1;
+}
 template <int ND, bool CART, int MODE, typename T>
-__global__ void k_lad_nodeflux_all(DevGrid g, const T* __restrict__ W, const T* __restrict__ bt,
+__global__ void __launch_bounds__(128, nodeflux_blocks<ND, T>()) k_lad_nodeflux_all(DevGrid g, const T* __restrict__ W, const T* __restrict__ bt,
                                    const T* __restrict__ kp, const T* __restrict__ gr, const T* __restrict__ dv, Box b3,
                                    const T* __restrict__ vco, Box vbx, T* __restrict__ F0, Box fb0, T* __restrict__ F1,
                                    Box fb1, T* __restrict__ F2, Box fb2, Box ub, const int* guard, int want) {
@@ -546,14 +568,6 @@ __global__ void k_lad_nodeflux_all(DevGrid g, const T* __restrict__ W, const T* 
       for (int v = 0; v < NV; ++v) Fo[v * fs + q] = F[l][v];
     }
   }
-}
-
-template <int ND, bool CART, int MODE, typename T = double>
-__global__ void k_lad_nodeflux(DevGrid g, int l, const T* __restrict__ W, const T* __restrict__ bt,
-                               const T* __restrict__ kp, const T* __restrict__ gr, const T* __restrict__ dv, Box b3,
-                               const T* __restrict__ vco, Box vbx, T* __restrict__ Fn, Box fb, const int* guard,
-                               int want) {
-  k_lad_nodeflux_body<ND, CART, MODE, T>(hw_block(), g, l, W, bt, kp, gr, dv, b3, vco, vbx, Fn, fb, guard, want);
 }
 
 // Physical viscosity of Eq. (3) with Sutherland's law at every node of vbx,
@@ -619,72 +633,60 @@ __device__ __forceinline__ void lad_epilogue(const DevGrid& g, const StageArgs& 
   stage_epilogue<ND, FUSED, TA>(g, A, qi, J, tot, out);
 }
 
-// E4 divergence of the node fluxes along l (explicit) or the compact result D.
+// The C6 divergence along l from its line buffer D (1D grids).
 template <int ND, typename T = double>
-__global__ void k_lad_div(DevGrid g, int l, const T* __restrict__ Fn, Box fb, const T* __restrict__ D,
-                          LineBuf DL, StageArgs A, const int* guard, int want) {
+__global__ void k_lad_div(DevGrid g, int l, const T* __restrict__ D, LineBuf DL, StageArgs A, const int* guard, int want) {
   constexpr int NV = ND + 2;
   if (guard && *guard != want) return;
-  long long fs = fb.size();
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < g.N; q += (long long)gridDim.x * blockDim.x) {
     int c[3];
     node_coords(g, q, c);
     T Dv[NV];
-    if (D) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) Dv[v] = D[DL.at(v, c[l], c)];
-    } else {
-      long long e = fb.at(c[0], c[1], c[2]);
-      long long st = l == 0 ? 1 : (l == 1 ? (long long)fb.ext[0] : (long long)fb.ext[0] * fb.ext[1]);
+    for (int v = 0; v < NV; ++v) Dv[v] = D[DL.at(v, c[l], c)];
+    lad_epilogue<ND, sizeof(T) == 4, T>(g, A, q, c, Dv);
+  }
+}
+
+// The E4 divergences of all directions in one pass (the node fluxes of each
+// direction in its own slice), summed in the order of the per-direction
+// launches in the accumulator's type, then one epilogue: the accumulator is not
+// written and read again between directions.
+template <int ND, typename T>
+__global__ void k_lad_div_all(DevGrid g, const T* __restrict__ F0, Box fb0, const T* __restrict__ F1, Box fb1,
+                              const T* __restrict__ F2, Box fb2, StageArgs A, const int* guard, int want) {
+  constexpr int NV = ND + 2;
+  using TA = typename std::conditional<sizeof(T) == 4, float, double>::type;
+  if (guard && *guard != want) return;
+  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < g.N; q += (long long)gridDim.x * blockDim.x) {
+    int c[3];
+    node_coords(g, q, c);
+    T Dv[NV];
+#pragma unroll
+    for (int l = 0; l < ND; ++l) {
+      const Box& fb = l == 0 ? fb0 : (l == 1 ? fb1 : fb2);
+      const T* Fn = l == 0 ? F0 : (l == 1 ? F1 : F2);
+      const long long e = fb.at(c[0], c[1], c[2]), fs = fb.size();
+      const long long st = l == 0 ? 1 : (l == 1 ? (long long)fb.ext[0] : (long long)fb.ext[0] * fb.ext[1]);
+      T d[NV];
       with_products<T>([&](auto P) {
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           const T* f = Fn + v * fs;
-          Dv[v] = d4(P, f[e - 2 * st], f[e - st], f[e + st], f[e + 2 * st]);
+          d[v] = d4(P, f[e - 2 * st], f[e - st], f[e + st], f[e + 2 * st]);
         }
       });
+#pragma unroll
+      for (int v = 0; v < NV; ++v) Dv[v] = l == 0 ? d[v] : T(TA(Dv[v]) + TA(d[v]));
     }
     lad_epilogue<ND, sizeof(T) == 4, T>(g, A, q, c, Dv);
   }
 }
 
-// The C6 divergence along x (D from the x-line buffer) on tiles of 32 (x) x
-// 8 lines: the tile's D values are staged with consecutive threads on
-// consecutive lines, then each thread takes one node, as k_lad_div.
-template <int ND, typename T>
-__global__ void __launch_bounds__(LGT_X * LGT_Y) k_lad_div_xt(DevGrid g, const T* __restrict__ D, LineBuf DL, StageArgs A,
-                                                            const int* guard, int want) {
-  constexpr int NV = ND + 2;
-  __shared__ T sD[NV][LGT_Y][LGT_X + 1];
-  if (guard && *guard != want) return;
-  const int x0 = (int)blockIdx.x * LGT_X;
-  const long long L0 = (long long)blockIdx.y * LGT_Y + (long long)blockIdx.z * gridDim.y * LGT_Y;
-  const int tid = threadIdx.y * LGT_X + threadIdx.x;
-  {
-    const int ly = tid % LGT_Y, lx = tid / LGT_Y;
-    if (x0 + lx < g.n[0] && L0 + ly < DL.nl) {
-      int c[3] = {0, 0, 0};
-      DL.coords(L0 + ly, c);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) sD[v][ly][lx] = D[DL.at(v, x0 + lx, c)];
-    }
-  }
-  __syncthreads();
-  const int x = x0 + (int)threadIdx.x;
-  const long long L = L0 + threadIdx.y;
-  if (x >= g.n[0] || L >= DL.nl) return;
-  int c[3] = {0, 0, 0};
-  DL.coords(L, c);
-  c[0] = x;
-  T Dv[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) Dv[v] = sD[v][threadIdx.y][threadIdx.x];
-  lad_epilogue<ND, sizeof(T) == 4, T>(g, A, lin(g, c[0], c[1], c[2]), c, Dv);
-}
-
-// The C6 divergences of all directions in one pass on the tiles of
-// k_lad_div_xt: the x derivatives staged through shared memory, the y (and z)
-// derivatives read directly, summed in the order of the per-direction
+// The C6 divergences of all directions in one pass on tiles of 32 (x) x 8
+// lines: the x derivatives staged through shared memory with consecutive
+// threads on consecutive lines (as k_lad_grad_xt), the y (and z) derivatives
+// read directly, summed in the order of the per-direction
 // launches (x, then y, then z, in the accumulator's type), then one epilogue.
 template <int ND, typename T>
 __global__ void __launch_bounds__(LGT_X * LGT_Y) k_lad_div_all_xt(DevGrid g, const T* __restrict__ D0, LineBuf DL0,
@@ -850,9 +852,16 @@ __device__ __forceinline__ void k_lad_hflux_body(const VBlock& vb, const DevGrid
   }
 }
 
-template <int ND, typename T = double>
-__global__ void k_lad_hflux(DevGrid g, int l, const T* __restrict__ Fn, Box fb, T* __restrict__ H, Box hb) {
-  k_lad_hflux_body<ND, T>(hw_block(), g, l, Fn, fb, H, hb);
+// The interface LAD fluxes of every direction in one launch (blockIdx.y: the direction).
+template <int ND, typename T>
+__global__ void k_lad_hflux_all(DevGrid g, const T* __restrict__ F0, Box fb0, T* __restrict__ H0, Box hb0,
+                                const T* __restrict__ F1, Box fb1, T* __restrict__ H1, Box hb1,
+                                const T* __restrict__ F2, Box fb2, T* __restrict__ H2, Box hb2) {
+  const VBlock vb{blockIdx.x, 0u, 0u, gridDim.x, 1u, 1u};
+  const int l = (int)blockIdx.y;
+  if (l == 0) k_lad_hflux_body<ND, T>(vb, g, 0, F0, fb0, H0, hb0);
+  if (ND > 1 && l == 1) k_lad_hflux_body<ND, T>(vb, g, 1, F1, fb1, H1, hb1);
+  if (ND > 2 && l == 2) k_lad_hflux_body<ND, T>(vb, g, 2, F2, fb2, H2, hb2);
 }
 
 }  // namespace cgk

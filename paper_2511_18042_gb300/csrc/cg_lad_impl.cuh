@@ -93,6 +93,8 @@ static int lad_coeffs_run(cg_solver* s, int dkind, cudaStream_t st, const int* g
   T* dv = reinterpret_cast<T*>(L.dv);
   T* bt[2] = {reinterpret_cast<T*>(L.bt[0]), reinterpret_cast<T*>(L.bt[1])};
   T* kp[2] = {reinterpret_cast<T*>(L.kp[0]), reinterpret_cast<T*>(L.kp[1])};
+  // the overbar's ND passes alternate between the two buffers: start where the last one ends in the first
+  int cur = ND & 1;
   k_lad_fieldbuf<ND, T><<<grid_blocks(L.fbx.size(), 256), 256, 0, st>>>(s->dg, reinterpret_cast<const T*>(s->W), fb, L.fbx);
   s->launches++;
   T* df[3] = {reinterpret_cast<T*>(L.df[0]), reinterpret_cast<T*>(L.df[1]), reinterpret_cast<T*>(L.df[2])};
@@ -125,7 +127,7 @@ static int lad_coeffs_run(cg_solver* s, int dkind, cudaStream_t st, const int* g
     else if (c6) k_lad_grad<ND, false, true, T><<<gb, 128, 0, st>>>(s->dg, fb, L.fbx, df[0], df[1], df[2], L.dfLB[0], L.dfLB[1], L.dfLB[2], gr, dv, L.b3, guard, want);
     else k_lad_grad<ND, false, false, T><<<gb, 128, 0, st>>>(s->dg, fb, L.fbx, df[0], df[1], df[2], L.dfLB[0], L.dfLB[1], L.dfLB[2], gr, dv, L.b3, guard, want);
     k_lad_coef<ND, false, T><<<grid_blocks(s->N, 128), 128, 0, st>>>(s->dg, reinterpret_cast<const T*>(s->W), fb, L.fbx, gr, dv, L.b3, s->p.c_beta,
-                                                                     s->p.c_kappa, bt[0], kp[0], guard, want);
+                                                                     s->p.c_kappa, bt[cur], kp[cur], guard, want);
   } else {
     if (xt) {
       if constexpr (ND >= 2)
@@ -135,38 +137,16 @@ static int lad_coeffs_run(cg_solver* s, int dkind, cudaStream_t st, const int* g
     else if (c6) k_lad_grad<ND, true, true, T><<<gb, 128, 0, st>>>(s->dg, fb, L.fbx, df[0], df[1], df[2], L.dfLB[0], L.dfLB[1], L.dfLB[2], gr, dv, L.b3, guard, want);
     else k_lad_grad<ND, true, false, T><<<gb, 128, 0, st>>>(s->dg, fb, L.fbx, df[0], df[1], df[2], L.dfLB[0], L.dfLB[1], L.dfLB[2], gr, dv, L.b3, guard, want);
     k_lad_coef<ND, true, T><<<grid_blocks(s->N, 128), 128, 0, st>>>(s->dg, reinterpret_cast<const T*>(s->W), fb, L.fbx, gr, dv, L.b3, s->p.c_beta,
-                                                                    s->p.c_kappa, bt[0], kp[0], guard, want);
+                                                                    s->p.c_kappa, bt[cur], kp[cur], guard, want);
   }
   s->launches += 2;
-  int cur = 0;
   for (int l = 0; l < ND; ++l) {
     k_gauss<ND, T><<<grid_blocks(s->N, 256), 256, 0, st>>>(s->dg, l, bt[cur], kp[cur], bt[1 - cur], kp[1 - cur],
                                                           guard, want);
     s->launches++;
     cur = 1 - cur;
   }
-  if (cur != 0) {
-    CG_CUDA(cudaMemcpyAsync(bt[0], bt[1], sizeof(T) * s->N, cudaMemcpyDeviceToDevice, st));
-    CG_CUDA(cudaMemcpyAsync(kp[0], kp[1], sizeof(T) * s->N, cudaMemcpyDeviceToDevice, st));
-  }
   return CG_OK;
-}
-
-template <int ND, int MODE, typename T>
-static void lad_nodeflux_m(cg_solver* s, int l, cudaStream_t st, const int* guard, int want, T* out) {
-  LadBuffers& L = s->lad;
-  int gb = grid_blocks(L.fbox[l].size(), 128);
-  const T* bt = reinterpret_cast<const T*>(L.bt[0]);
-  const T* kp = reinterpret_cast<const T*>(L.kp[0]);
-  const T* gr = reinterpret_cast<const T*>(L.gr);
-  const T* dv = reinterpret_cast<const T*>(L.dv);
-  T* Fn = out ? out : reinterpret_cast<T*>(L.Fn);
-  const T* vco = reinterpret_cast<const T*>(L.vco);
-  if (s->dg.curv)
-    k_lad_nodeflux<ND, false, MODE, T><<<gb, 128, 0, st>>>(s->dg, l, reinterpret_cast<const T*>(s->W), bt, kp, gr, dv, L.b3, vco, L.vbx, Fn, L.fbox[l], guard, want);
-  else
-    k_lad_nodeflux<ND, true, MODE, T><<<gb, 128, 0, st>>>(s->dg, l, reinterpret_cast<const T*>(s->W), bt, kp, gr, dv, L.b3, vco, L.vbx, Fn, L.fbox[l], guard, want);
-  s->launches++;
 }
 
 // mu, lambda, kappa of the physical viscosity at the nodes of every node flux
@@ -184,18 +164,9 @@ static void lad_viscoef(cg_solver* s, cudaStream_t st, const int* guard, int wan
   s->launches++;
 }
 
-// node fluxes along l: mode NF_LAD (artificial terms only), NF_LAD_VISC (plus
-// the physical viscosity) or NF_VISC (the physical viscous flux alone)
-// (out: where the fluxes go, the shared node-flux buffer when null)
-template <int ND, typename T = double>
-static void lad_nodeflux(cg_solver* s, int l, cudaStream_t st, const int* guard, int want, int mode = NF_LAD,
-                         T* out = nullptr) {
-  if (mode == NF_VISC) lad_nodeflux_m<ND, NF_VISC, T>(s, l, st, guard, want, out);
-  else if (mode == NF_LAD_VISC) lad_nodeflux_m<ND, NF_LAD_VISC, T>(s, l, st, guard, want, out);
-  else lad_nodeflux_m<ND, NF_LAD, T>(s, l, st, guard, want, out);
-}
-
-// node fluxes of every direction in one launch (k_lad_nodeflux_all), into out[l]
+// node fluxes of every direction in one launch (k_lad_nodeflux_all), into out[l]:
+// mode NF_LAD (artificial terms only), NF_LAD_VISC (plus the physical
+// viscosity) or NF_VISC (the physical viscous flux alone)
 template <int ND, int MODE, typename T>
 static void lad_nodeflux_all_m(cg_solver* s, cudaStream_t st, const int* guard, int want, T* const* out) {
   LadBuffers& L = s->lad;
@@ -219,8 +190,24 @@ static void lad_nodeflux_all_m(cg_solver* s, cudaStream_t st, const int* guard, 
 
 template <int ND, typename T>
 static void lad_nodeflux_all(cg_solver* s, cudaStream_t st, const int* guard, int want, int mode, T* const* out) {
-  if (mode == NF_LAD_VISC) lad_nodeflux_all_m<ND, NF_LAD_VISC, T>(s, st, guard, want, out);
+  if (mode == NF_VISC) lad_nodeflux_all_m<ND, NF_VISC, T>(s, st, guard, want, out);
+  else if (mode == NF_LAD_VISC) lad_nodeflux_all_m<ND, NF_LAD_VISC, T>(s, st, guard, want, out);
   else lad_nodeflux_all_m<ND, NF_LAD, T>(s, st, guard, want, out);
+}
+
+// the directions' slices of the node-flux buffer
+template <int ND, typename T>
+static void flux_slices(cg_solver* s, T** F) {
+  for (int l = 0; l < 3; ++l) F[l] = reinterpret_cast<T*>(s->lad.Fn) + (l < ND ? (size_t)l * s->lad.fstride : 0);
+}
+
+// E4 divergences of the node fluxes F of every direction with the epilogue of A
+template <int ND, typename T>
+static void lad_div_e4(cg_solver* s, T* const* F, const StageArgs& A, cudaStream_t st, const int* guard, int want) {
+  LadBuffers& L = s->lad;
+  k_lad_div_all<ND, T><<<grid_blocks(s->N, 256), 256, 0, st>>>(s->dg, F[0], L.fbox[0], F[1], L.fbox[ND > 1 ? 1 : 0], F[2],
+                                                              L.fbox[ND > 2 ? 2 : 0], A, guard, want);
+  s->launches++;
 }
 
 // E4 gradients of the LAD fields of the primitives in s->W (no coefficients)
@@ -247,17 +234,14 @@ static void lad_grad_e4(cg_solver* s, cudaStream_t st, const int* guard, int wan
 // the gradients of this stage's primitives are already in the LAD buffers.
 template <int ND, typename T>
 static void visc_pass(cg_solver* s, StageArgs A, cudaStream_t st, bool have_grad, const int* guard, int want) {
-  LadBuffers& L = s->lad;
   if (!have_grad) lad_grad_e4<ND, T>(s, st, guard, want);
   lad_viscoef<ND, T>(s, st, guard, want, false);
-  for (int l = 0; l < ND; ++l) {
-    lad_nodeflux<ND, T>(s, l, st, guard, want, NF_VISC);
-    A.first = l == 0;
-    A.last = false;
-    k_lad_div<ND, T><<<grid_blocks(s->N, 256), 256, 0, st>>>(s->dg, l, reinterpret_cast<const T*>(L.Fn), L.fbox[l],
-                                                            nullptr, L.DLB[l], A, guard, want);
-    s->launches++;
-  }
+  T* F[3];
+  flux_slices<ND, T>(s, F);
+  lad_nodeflux_all<ND, T>(s, st, guard, want, NF_VISC, F);
+  A.first = true;
+  A.last = false;
+  lad_div_e4<ND, T>(s, F, A, st, guard, want);
 }
 
 template <int ND>
@@ -312,27 +296,19 @@ static int lad_pass(cg_solver* s, int dkind, StageArgs A, cudaStream_t st, const
     s->launches++;
     return CG_OK;
   }
-  // E4: every direction's node fluxes in one pass too (slices of Fn)
-  T* Fe[3] = {nullptr, nullptr, nullptr};
-  if (dkind != 3) {
-    for (int l = 0; l < ND; ++l) Fe[l] = reinterpret_cast<T*>(L.Fn) + (size_t)l * L.fstride;
-    lad_nodeflux_all<ND, T>(s, st, guard, want, nfm, Fe);
+  if (dkind != 3) {  // E4: every direction's node fluxes and divergences in one pass each
+    T* F[3];
+    flux_slices<ND, T>(s, F);
+    lad_nodeflux_all<ND, T>(s, st, guard, want, nfm, F);
+    A.first = true;
+    A.last = true;
+    lad_div_e4<ND, T>(s, F, A, st, guard, want);
+    return CG_OK;
   }
-  for (int l = 0; l < ND; ++l) {
+  for (int l = 0; l < ND; ++l) {  // C6 in 1D
     A.first = l == 0;
     A.last = l == ND - 1;
-    const T* D = Dl[l];
-    LineBuf DL = L.DLB[l];
-    if (ND >= 2 && l == 0 && D) {  // x lines: the tiled read of the line buffer
-      const long long ty = (DL.nl + LGT_Y - 1) / LGT_Y;
-      const unsigned gy = (unsigned)std::min<long long>(ty, 65535), gz = (unsigned)((ty + gy - 1) / gy);
-      if constexpr (ND >= 2)
-        k_lad_div_xt<ND, T><<<dim3((unsigned)((s->dg.n[0] + LGT_X - 1) / LGT_X), gy, gz), dim3(LGT_X, LGT_Y), 0, st>>>(
-            s->dg, D, DL, A, guard, want);
-    } else {
-      k_lad_div<ND, T><<<grid_blocks(s->N, 256), 256, 0, st>>>(s->dg, l, Fe[l] ? Fe[l] : reinterpret_cast<const T*>(L.Fn),
-                                                              L.fbox[l], D, DL, A, guard, want);
-    }
+    k_lad_div<ND, T><<<grid_blocks(s->N, 256), 256, 0, st>>>(s->dg, l, Dl[l], L.DLB[l], A, guard, want);
     s->launches++;
   }
   return CG_OK;
@@ -353,8 +329,7 @@ static int lad_stage_t(cg_solver* s, const double* Uc, StageArgs A, cudaStream_t
   launch_prim<ND>(s, Uc, st);  // T is the precision's type
   if (sch == CG_LAD_E4 || sch == CG_LAD_C6) return lad_pass<ND, T>(s, sch == CG_LAD_E4 ? 2 : 3, A, st, nullptr, 0);
   LadBuffers& L = s->lad;
-  CG_CUDA(cudaMemsetAsync(s->hyb_flag, 0, sizeof(int), st));
-  CG_CUDA(cudaMemsetAsync(s->hyb_count, 0, sizeof(unsigned long long), st));
+  CG_CUDA(cudaMemsetAsync(s->hyb_count, 0, 2 * sizeof(unsigned long long), st));  // the count and the flag behind it
   if (s->p.hybrid_mode == CG_HYBRID_GLOBAL) {
     // Algorithm 3: GBR-MEG6 for the whole stage if any node is troubled, else LAD-E4
     k_troubled<ND, T><<<grid_blocks(L.tbox.size(), 256), 256, 0, st>>>(s->dg, reinterpret_cast<const T*>(s->W), s->p.hyb_rho, s->p.hyb_p, nullptr,
@@ -379,12 +354,18 @@ static int lad_stage_t(cg_solver* s, const double* Uc, StageArgs A, cudaStream_t
   int rc = lad_coeffs_run<ND, T>(s, 2, st, nullptr, 0);
   if (rc) return rc;
   if (s->p.viscous) visc_pass<ND, T>(s, A, st, true, nullptr, 0);
-  for (int l = 0; l < ND; ++l) {
-    lad_nodeflux<ND, T>(s, l, st, nullptr, 0);
-    k_lad_hflux<ND, T><<<grid_blocks(L.hbox[l].size(), 256), 256, 0, st>>>(s->dg, l, reinterpret_cast<const T*>(L.Fn),
-                                                                          L.fbox[l], reinterpret_cast<T*>(s->hflux[l]), L.hbox[l]);
-    s->launches++;
+  T *F[3], *Hf[3];
+  flux_slices<ND, T>(s, F);
+  lad_nodeflux_all<ND, T>(s, st, nullptr, 0, NF_LAD, F);
+  long long hmax = 0;
+  for (int l = 0; l < 3; ++l) {
+    Hf[l] = reinterpret_cast<T*>(s->hflux[l < ND ? l : 0]);
+    hmax = std::max(hmax, (long long)L.hbox[l < ND ? l : 0].size());
   }
+  k_lad_hflux_all<ND, T><<<dim3((unsigned)grid_blocks(hmax, 256), ND), 256, 0, st>>>(
+      s->dg, F[0], L.fbox[0], Hf[0], L.hbox[0], F[1], L.fbox[ND > 1 ? 1 : 0], Hf[1], L.hbox[ND > 1 ? 1 : 0], F[2],
+      L.fbox[ND > 2 ? 2 : 0], Hf[2], L.hbox[ND > 2 ? 2 : 0]);
+  s->launches++;
   StageArgs H = A;
   H.mask = L.tr;
   H.tBox = L.tbox;

@@ -742,8 +742,17 @@ struct XTileFilter {
   __device__ void load(const int* c, double* w) const { load_filtered<ND>(g, U, c, w); }
   __device__ double row(const double* w, int p, bool closure) const {
     if (closure) return w[p];
-    return b0 * w[p] + b1 * (w[p + 1] + w[p - 1]) + b2 * (w[p + 2] + w[p - 2]) + b3 * (w[p + 3] + w[p - 3]) +
-           b4 * (w[p + 4] + w[p - 4]);
+    double r;
+    with_products<double>([&](auto P) {
+      require_range(P, b0);
+      require_range(P, b1);
+      require_range(P, b2);
+      require_range(P, b3);
+      require_range(P, b4);
+      r = P.kz(b0, w[p]) + P.kz(b1, w[p + 1] + w[p - 1]) + P.kz(b2, w[p + 2] + w[p - 2]) +
+          P.kz(b3, w[p + 3] + w[p - 3]) + P.kz(b4, w[p + 4] + w[p - 4]);
+    });
+    return r;
   }
 };
 
