@@ -201,13 +201,9 @@ static int table_build_t(BatchTable& tb, cg_solver* const* sv, double* const* st
     JobOmega<T> o;
     o.g = s->dg;
     o.W = W;
-    for (int d = 0; d < 3; ++d) {
-      o.G[d] = reinterpret_cast<const T*>(s->G[d]);
-      o.gb[d] = s->gdLB[d];
-    }
     o.om = reinterpret_cast<T*>(s->om);
     o.ob = s->omBox;
-    o.nb = (unsigned)table_blocks(s->omBox.size());
+    o.gx = (unsigned)((s->omBox.ext[0] + OMT_X - 1) / OMT_X);
     om[m] = o;
     fd[m] = JobField<T>{s->dg, W, fb, L.fbx, (unsigned)table_blocks(L.fbx.size())};
     tr[m] = JobTroubled<T>{s->dg, W, s->p.hyb_rho, s->p.hyb_p, s->p.hybrid_sensor ? reinterpret_cast<const T*>(s->om) : nullptr, s->omBox,
@@ -235,7 +231,7 @@ static int table_build_t(BatchTable& tb, cg_solver* const* sv, double* const* st
                              (unsigned)table_blocks(L.hbox[l].size())};
     }
   }
-  blob.add(&tb.omega, om, offsets([&](int m) { return (long long)om[m].nb; }));
+  blob.add(&tb.omega, om, offsets([&](int m) { return om[m].blocks(); }));
   blob.add(&tb.field, fd, offsets([&](int m) { return (long long)fd[m].nb; }));
   blob.add(&tb.troubled, tr, offsets([&](int m) { return (long long)tr[m].nb; }));
   blob.add(&tb.grad, gr, offsets([&](int m) { return (long long)gr[m].nb; }));

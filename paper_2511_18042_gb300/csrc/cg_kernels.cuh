@@ -411,18 +411,17 @@ __global__ void k_omega(DevGrid g, const T* __restrict__ W, const T* __restrict_
 // 256 x 96 x 64 instead of 1.89 at two.)
 constexpr int OMT_X = 32, OMT_Y = 8, OMT_H = 3;
 template <int ND, bool CART, typename T>
-__global__ void __launch_bounds__(OMT_X * OMT_Y, ND == 3 && sizeof(T) == 8 ? 3 : 1) k_omega_tile(DevGrid g, const T* __restrict__ W, T* __restrict__ om, Box ob,
-                                                             const int* guard, int want) {
+__device__ __forceinline__ void k_omega_tile_body(const VBlock& vb, const DevGrid& g, const T* __restrict__ W,
+                                                  T* __restrict__ om, const Box& ob) {
   static_assert(ND >= 2, "tiles of x and y");
   constexpr int NV = ND + 2, IP = ND + 1;
   constexpr int SX = OMT_X + 2 * OMT_H, SY = OMT_Y + 2 * OMT_H;
   __shared__ T sP[SY][SX];
   __shared__ T sU[ND][SY][SX];
-  if (guard && *guard != want) return;
-  const int x0 = (int)blockIdx.x * OMT_X - ob.off[0], y0 = (int)blockIdx.y * OMT_Y - ob.off[1];
-  const int cz = ND == 3 ? (int)blockIdx.z - ob.off[2] : 0;
+  const int x0 = (int)vb.x * OMT_X - ob.off[0], y0 = (int)vb.y * OMT_Y - ob.off[1];
+  const int cz = ND == 3 ? (int)vb.z - ob.off[2] : 0;
   const bool zin = cz >= 0 && cz < (ND == 3 ? g.n[2] : 1);
-  const int tid = threadIdx.y * OMT_X + threadIdx.x;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x, lx = tid % OMT_X, ly = tid / OMT_X;
   for (int e = tid; e < SX * SY; e += OMT_X * OMT_Y) {
     const int sy = e / SX, sx = e - sy * SX;
     const int x = x0 - OMT_H + sx, y = y0 - OMT_H + sy;
@@ -439,10 +438,10 @@ __global__ void __launch_bounds__(OMT_X * OMT_Y, ND == 3 && sizeof(T) == 8 ? 3 :
     for (int k = 0; k < ND; ++k) sU[k][sy][sx] = w[1 + k];
   }
   __syncthreads();
-  const int ex = (int)blockIdx.x * OMT_X + threadIdx.x, ey = (int)blockIdx.y * OMT_Y + threadIdx.y;
+  const int ex = (int)vb.x * OMT_X + lx, ey = (int)vb.y * OMT_Y + ly;
   if (ex >= ob.ext[0] || ey >= ob.ext[1]) return;
-  int c[3] = {x0 + (int)threadIdx.x, y0 + (int)threadIdx.y, cz};
-  const int tx = threadIdx.x + OMT_H, ty = threadIdx.y + OMT_H;
+  int c[3] = {x0 + lx, y0 + ly, cz};
+  const int tx = lx + OMT_H, ty = ly + OMT_H;
   const T p0 = sP[ty][tx];
   T phi = T(0);
   phi = raise_to(phi, sensor_phi<T>(sP[ty][tx - 1], p0, sP[ty][tx + 1]));
@@ -479,6 +478,13 @@ __global__ void __launch_bounds__(OMT_X * OMT_Y, ND == 3 && sizeof(T) == 8 ? 3 :
     sensor_gu<ND, CART, T>(P, g, c, du, gu);
   });
   om[ob.at(c[0], c[1], c[2])] = phi * sensor_zeta<ND, T>(gu);
+}
+
+template <int ND, bool CART, typename T>
+__global__ void __launch_bounds__(OMT_X * OMT_Y, ND == 3 && sizeof(T) == 8 ? 3 : 1) k_omega_tile(DevGrid g, const T* __restrict__ W, T* __restrict__ om, Box ob,
+                                                             const int* guard, int want) {
+  if (guard && *guard != want) return;
+  k_omega_tile_body<ND, CART, T>(hw_block(), g, W, om, ob);
 }
 
 // ---------------------------------------------------------------- compact gradients

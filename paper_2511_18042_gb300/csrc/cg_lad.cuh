@@ -377,6 +377,53 @@ __global__ void k_gauss(DevGrid g, int l, const T* __restrict__ a, const T* __re
   k_gauss_body<ND, T>(hw_block(), g, l, a, b, ao, bo, guard, want);
 }
 
+// Both passes of the overbar of a 2D grid in one: a block filters the rows of
+// its tile and of a halo of four along x (a ghost row is the row the boundary
+// rule names, as k_gauss reads it), holds them in shared memory and filters
+// along y.  Same values as two k_gauss passes (58 us a step of the triple point
+// 1792 x 768 instead of 85).  FP32 only: the halo's rows are filtered twice, which
+// costs an FP64-bound kernel more than the pass over memory.
+constexpr int GT_X = 32, GT_Y = 16;
+template <typename T>
+__global__ void __launch_bounds__(256) k_gauss2_tile(DevGrid g, const T* __restrict__ a, const T* __restrict__ b,
+                                                   T* __restrict__ ao, T* __restrict__ bo, const int* guard, int want) {
+  constexpr int R = GT_Y + 8;
+  __shared__ T sa[R][GT_X], sb[R][GT_X];
+  if (guard && *guard != want) return;
+  const T A0 = T(3565.0 / 10368.0), A1 = T(3091.0 / 12960.0), A2 = T(1997.0 / 25920.0), A3 = T(149.0 / 12960.0),
+          A4 = T(107.0 / 103680.0);
+  const int lx = threadIdx.x % GT_X, x = (int)blockIdx.x * GT_X + lx, y0 = (int)blockIdx.y * GT_Y;
+  const int n0 = g.n[0], n1 = g.n[1];
+  if (x < n0) {
+    for (int r = threadIdx.x / GT_X; r < R && y0 - 4 + r < n1 + 4; r += 256 / GT_X) {
+      const long long row = scalar_src(g, 0, y0 - 4 + r, 0);  // node 0 of the row (the boundary rules are separable)
+      long long s[9];
+      if (x >= 4 && x < n0 - 4) {
+#pragma unroll
+        for (int t = -4; t <= 4; ++t) s[t + 4] = row + x + t;
+      } else {
+#pragma unroll
+        for (int t = -4; t <= 4; ++t) s[t + 4] = row + scalar_src(g, x + t, 0, 0);
+      }
+      sa[r][lx] = A0 * a[s[4]] + A1 * (a[s[3]] + a[s[5]]) + A2 * (a[s[2]] + a[s[6]]) + A3 * (a[s[1]] + a[s[7]]) +
+                  A4 * (a[s[0]] + a[s[8]]);
+      sb[r][lx] = A0 * b[s[4]] + A1 * (b[s[3]] + b[s[5]]) + A2 * (b[s[2]] + b[s[6]]) + A3 * (b[s[1]] + b[s[7]]) +
+                  A4 * (b[s[0]] + b[s[8]]);
+    }
+  }
+  __syncthreads();
+  if (x >= n0) return;
+  for (int ry = threadIdx.x / GT_X; ry < GT_Y && y0 + ry < n1; ry += 256 / GT_X) {
+    auto overbar = [&](const T(&f)[R][GT_X]) {
+      return A0 * f[ry + 4][lx] + A1 * (f[ry + 3][lx] + f[ry + 5][lx]) + A2 * (f[ry + 2][lx] + f[ry + 6][lx]) +
+             A3 * (f[ry + 1][lx] + f[ry + 7][lx]) + A4 * (f[ry][lx] + f[ry + 8][lx]);
+    };
+    const long long q = lin(g, x, y0 + ry, 0);
+    ao[q] = overbar(sa);
+    bo[q] = overbar(sb);
+  }
+}
+
 // Node fluxes along l at positions [-2, n+1] (interior lines).
 // MODE 0 (LAD, inviscid case): F = F^c(W; xi_hat_l) - [0, xi_hat_l tau,
 //   xi_hat_l . phi], tau = beta* div, phi_m = u_m tau + kappa* dT/dx_m.
@@ -411,30 +458,10 @@ __device__ __forceinline__ void nodeflux_at(const DevGrid& g, int l, const T* __
     }
     const T rho = w[0], p = w[IP];
     const long long be = b3.at(c[0], c[1], c[2]);
-    const T div = dv[be];
     auto G = [&](int f, int m) { return gr[(f * ND + m) * bs + be]; };
-    [[maybe_unused]] T tau1, kap, mu, lam;
-    if constexpr (PHYS) {
-      // mu, lambda = beta* - 2/3 mu and kappa* + mu / ((gamma-1) Pr M^2) of
-      // the node, formed once per stage by k_lad_viscoef
-      const long long vq = vbx.at(c[0], c[1], c[2]), vs = vbx.size();
-      mu = vco[vq];
-      lam = vco[vs + vq];
-      kap = vco[2 * vs + vq];
-    } else {
-      const long long sq = scalar_src(g, c[0], c[1], c[2]);
-      tau1 = bt[sq] * div;
-      kap = kp[sq];
-    }
-    T pg = T(0);  // p / (gamma - 1)
-    if (CONV) pg = div_t(p, gconst<T>(g.gm1, g.f_gm1));
     with_products<T>([&](auto P) {
       if (CART) require_range(P, xi[l]);
       if (CONV) require_range(P, rho);
-      if (PHYS) {
-        require_range(P, mu);
-        require_range(P, kap);
-      }
       auto X = [&](T a, T b) { return CART ? P.kz(a, b) : P.zz(a, b); };  // by a metric component
       if (CONV) {
         T U, q2;
@@ -447,7 +474,7 @@ __device__ __forceinline__ void nodeflux_at(const DevGrid& g, int l, const T* __
         q2 = w[1] * w[1];
 #pragma unroll
         for (int m = 1; m < ND; ++m) q2 = q2 + w[1 + m] * w[1 + m];
-        const T E = add_scaled(pg, T(0.5), P.kz(rho, q2));
+        const T E = add_scaled(div_t(p, gconst<T>(g.gm1, g.f_gm1)), T(0.5), P.kz(rho, q2));
         F[0] = P.kz(rho, U);
 #pragma unroll
         for (int m = 0; m < ND; ++m) {
@@ -462,6 +489,8 @@ __device__ __forceinline__ void nodeflux_at(const DevGrid& g, int l, const T* __
       T fe = T(0);
       bool first = true;
       if constexpr (!PHYS) {
+        const long long sq = scalar_src(g, c[0], c[1], c[2]);
+        const T tau1 = bt[sq] * dv[be], kap = kp[sq];
 #pragma unroll
         for (int m = 0; m < ND; ++m) {
           if (CART && m != l) continue;
@@ -474,6 +503,12 @@ __device__ __forceinline__ void nodeflux_at(const DevGrid& g, int l, const T* __
           if (!CART || m == l) F[1 + m] = F[1 + m] - X(xi[m], tau1);
         F[IP] = F[IP] - fe;
       } else {
+        // mu, lambda = beta* - 2/3 mu and kappa* + mu / ((gamma-1) Pr M^2) of
+        // the node, formed once per stage by k_lad_viscoef
+        const long long vq = vbx.at(c[0], c[1], c[2]), vs = vbx.size();
+        const T mu = vco[vq], lam = vco[vs + vq], kap = vco[2 * vs + vq], div = dv[be];
+        require_range(P, mu);
+        require_range(P, kap);
         T tau[ND][ND];
 #pragma unroll
         for (int m = 0; m < ND; ++m)
@@ -539,10 +574,11 @@ __device__ __forceinline__ bool box_holds(const Box& b, const int* c) {
 
 // Blocks an SM (of 128 threads): the 3D FP64 form would take 190 registers; held
 // to 128 the viscous node fluxes of the 3D ramp 256 x 96 x 64 take 1.58 ms a step
-// instead of 1.79 (1.86 with a launch for each direction).
+// instead of 1.79 (1.86 with a launch for each direction).  FP32: bound by
+// latency, 64 registers in 3D and 40 below.
 template <int ND, typename T>
 __host__ __device__ constexpr int nodeflux_blocks() {
-  return ND == 3 && sizeof(T) == 8 ? 4 : 1;
+  return sizeof(T) == 8 ? (ND == 3 ? 4 : 1) : (ND == 3 ? 8 : 12);
 }
 template <int ND, bool CART, int MODE, typename T>
 __global__ void __launch_bounds__(128, nodeflux_blocks<ND, T>()) k_lad_nodeflux_all(DevGrid g, const T* __restrict__ W, const T* __restrict__ bt,

@@ -94,7 +94,9 @@ static int lad_coeffs_run(cg_solver* s, int dkind, cudaStream_t st, const int* g
   T* bt[2] = {reinterpret_cast<T*>(L.bt[0]), reinterpret_cast<T*>(L.bt[1])};
   T* kp[2] = {reinterpret_cast<T*>(L.kp[0]), reinterpret_cast<T*>(L.kp[1])};
   // the overbar's ND passes alternate between the two buffers: start where the last one ends in the first
-  int cur = ND & 1;
+  // (a 2D FP32 overbar is one pass)
+  constexpr bool gauss2 = ND == 2 && sizeof(T) == 4;
+  int cur = gauss2 ? 1 : ND & 1;
   k_lad_fieldbuf<ND, T><<<grid_blocks(L.fbx.size(), 256), 256, 0, st>>>(s->dg, reinterpret_cast<const T*>(s->W), fb, L.fbx);
   s->launches++;
   T* df[3] = {reinterpret_cast<T*>(L.df[0]), reinterpret_cast<T*>(L.df[1]), reinterpret_cast<T*>(L.df[2])};
@@ -140,6 +142,12 @@ static int lad_coeffs_run(cg_solver* s, int dkind, cudaStream_t st, const int* g
                                                                     s->p.c_kappa, bt[cur], kp[cur], guard, want);
   }
   s->launches += 2;
+  if constexpr (gauss2) {
+    const dim3 grid((unsigned)((s->dg.n[0] + GT_X - 1) / GT_X), (unsigned)((s->dg.n[1] + GT_Y - 1) / GT_Y));
+    k_gauss2_tile<T><<<grid, 256, 0, st>>>(s->dg, bt[1], kp[1], bt[0], kp[0], guard, want);
+    s->launches++;
+    return CG_OK;
+  }
   for (int l = 0; l < ND; ++l) {
     k_gauss<ND, T><<<grid_blocks(s->N, 256), 256, 0, st>>>(s->dg, l, bt[cur], kp[cur], bt[1 - cur], kp[1 - cur],
                                                           guard, want);
