@@ -164,6 +164,8 @@ def run(requests, budget_bytes=100 << 30, precision=1, device="cuda", max_active
             if inflight:
                 retire(inflight.popleft())
                 continue
+            if not pending:  # the last tick was retired at the head of this pass
+                continue
             wait = pending[0].arrival - (time.perf_counter() - t0)
             if wait > 0:
                 time.sleep(min(wait, 0.05))

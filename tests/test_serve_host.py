@@ -81,3 +81,51 @@ def test_state_bytes_and_solver_kwargs():
         assert serve.state_bytes(r.prob) == 8 * nv * r.cells == r.prob["U"].nbytes
         kw = serve.solver_kwargs(r.prob)
         assert kw["hybrid_mode"] == 1 and kw["hybrid_buffer"] == 1 and kw["precision"] == 1
+
+
+class _DoneEvent:
+    """An event that has completed by the time it is asked about."""
+
+    def __init__(self, enable_timing=False):
+        pass
+
+    def record(self, stream=None):
+        pass
+
+    def query(self):
+        return True
+
+    def synchronize(self):
+        pass
+
+    def elapsed_time(self, other):
+        return 0.0
+
+
+def test_loop_ends_when_the_last_tick_completes_at_once(monkeypatch):
+    """Ticks that are complete when the loop comes back to them (short steps, a
+    slow host): the last one is retired before anything looks for pending work."""
+    import contextlib
+    import torch
+
+    class Solver:
+        @classmethod
+        def from_problem(cls, prob, **kw):
+            return cls()
+
+        def device_bytes(self):
+            return 1
+
+        def sync_status(self, stream):
+            return 0
+
+    empty = torch.empty
+    monkeypatch.setattr(torch.cuda, "Event", _DoneEvent)
+    monkeypatch.setattr(torch.cuda, "Stream", lambda dev=None: None)
+    monkeypatch.setattr(torch.cuda, "stream", lambda s: contextlib.nullcontext())
+    monkeypatch.setattr(torch, "empty", lambda *a, pin_memory=False, **kw: empty(*a, **kw))
+    monkeypatch.setattr(serve.api, "Solver", Solver)
+    monkeypatch.setattr(serve.api, "multi_step", lambda solvers, states, stream=None: None)
+    reqs = serve.request_mix(3, rate=1e6, seed=1, tube=(20, 40), steps=(2, 4), frac_tube=1.0)
+    stats, done = serve.run(reqs, device="cpu")
+    assert stats["ok"] == 3 and sorted(r.rid for r in done) == [0, 1, 2]
