@@ -91,7 +91,7 @@ typedef struct {
     double twall;         /* temperature of CG_BC_WALL faces (units of T_inf) */
     /* FP64 C-GBR interface sweep.  0 (default): every expression in the
      * oracle's operation order, no a*b+c contracted (bitwise reproducible).
-     * 1: multiply-adds fused (16 % fewer FP64 instructions in the sweep);
+     * 1: multiply-adds fused instead of products on the integer pipes;
      * results agree to rounding, except where a value sits at a threshold of
      * the selection (Eq. 8) and the branch flips: on the 1792x768 triple point
      * the per-interface hybrid then differs by ~1e-11 after one step.  Other

@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(256) k_gauss2_tile(DevGrid g, const T* __restr
 // (MODE 2: no convective flux, beta* = kappa* = 0).
 constexpr int NF_LAD = 0, NF_LAD_VISC = 1, NF_VISC = 2;
 
-// node flux along l at node c (the body of k_lad_nodeflux; F: nv values)
+// node flux along l at node c (F: nv values)
 template <int ND, bool CART, int MODE, typename T>
 __device__ __forceinline__ void nodeflux_at(const DevGrid& g, int l, const T* __restrict__ W, const T* __restrict__ bt,
                                             const T* __restrict__ kp, const T* __restrict__ gr,
@@ -566,7 +566,7 @@ __device__ __forceinline__ void k_lad_nodeflux_body(const VBlock& vb, const DevG
 // The node fluxes of every direction in one pass over ub (the union of the
 // directions' boxes, positions [-2, n+1] in every direction): each node forms
 // all directions' fluxes (the loads they share, issued once) and stores those
-// whose box holds it; the values are those of k_lad_nodeflux.
+// whose box holds it.
 __device__ __forceinline__ bool box_holds(const Box& b, const int* c) {
   return c[0] + b.off[0] >= 0 && c[0] + b.off[0] < b.ext[0] && c[1] + b.off[1] >= 0 && c[1] + b.off[1] < b.ext[1] &&
          c[2] + b.off[2] >= 0 && c[2] + b.off[2] < b.ext[2];
