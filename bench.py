@@ -685,6 +685,8 @@ def sweep_roofline(api, torch, grid, base, dev, args, peaks):
     ach = SWEEP_FLOP_PER_IFACE * ifaces / (avg_ms * 1e-3) / 1e12
     roof.update({"achieved": ach, "frac": ach / peak, "algorithmic_flop_per_iface": SWEEP_FLOP_PER_IFACE,
                  "flop_source": "oracle operation count (profiles/flops_triple_point_1792x768.md)",
+                 "frac_note": "divisions, roots, comparisons and products with a known factor run on the integer "
+                              "and FP32 pipes: the counted operations per time may exceed the FP64 pipe's peak",
                  "peak_measured": {k: v for k, v in peaks.items() if k != "clocks"}})
     fms, fn, ftile = _sweep_ms(api, torch, grid, base, dev, args, "contracted")
     fach = SWEEP_FLOP_PER_IFACE * ifaces / (fms * 1e-3) / 1e12
