@@ -424,8 +424,10 @@ __device__ __forceinline__ void hllc_f64(const PR& P, const GbrCfg& q, const dou
     R.any(den);
     Ss = div_by(num, divisor(den));
   }
+  // the first of 0 <= SL, 0 <= S*, 0 <= SR that holds decides (S* may exceed SR
+  // where gamma is near 1)
   const bool left = nonneg(SL) || nonneg(Ss);
-  const bool star = !nonneg(SL) && nonneg(SR);
+  const bool star = !nonneg(SL) && (nonneg(Ss) || nonneg(SR));
   double W[ND];
 #pragma unroll
   for (int m = 0; m < ND; ++m) W[m] = left ? WL[1 + m] : WR[1 + m];

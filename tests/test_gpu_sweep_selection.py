@@ -1,0 +1,54 @@
+"""The choices of the FP64 interface sweep (HLLC state, sensor window) in the
+corners where a shortened test could choose differently, against the oracle
+(1e-13 of each variable's largest magnitude for one RHS evaluation)."""
+import numpy as np
+import pytest
+
+from paper_2511_18042_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+from tests.gpu_util import rel_err, to_dev  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def api():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2511_18042_gb300 import api as a
+    return a
+
+
+@pytest.mark.parametrize("fma", [0, 1])
+@pytest.mark.parametrize("gamma", [1.001, 1.000001])
+def test_contact_right_of_the_right_wave(orc, api, gamma, fma):
+    """gamma near 1 and a strong jump: the estimated contact speed can exceed
+    the right wave's, SR < 0 <= S*.  The flux there is the left star state's
+    (the first test of Eq. (10) that holds decides)."""
+    rL, pL, rR = 95.6224235889941, 6034.428430832117, 0.014406564806903267
+    c = np.sqrt(gamma * pL / rL)
+    jumps = []
+    for pR in (4e-3, 1e-3, 1e-4):
+        for d in np.linspace(-2e-3, 6e-3, 33):
+            jumps.append((pR, -c * (1.0 + d)))
+    N = 16 * len(jumps)
+    W = np.empty((3, N))
+    for k, (pR, u) in enumerate(jumps):
+        W[:, 16 * k:16 * k + 8] = np.array([rL, u, pL])[:, None]
+        W[:, 16 * k + 8:16 * k + 16] = np.array([rR, u, pR])[:, None]
+    prob = inputs._problem("jumps", 1, [N], [1.0], [[inputs.EXTRAP, inputs.EXTRAP]], W, gamma)
+    # the waves of the cell states at every jump from the dense to the thin gas
+    gm1 = gamma - 1.0
+    pR, u = np.array(jumps).T
+    H = [(p / gm1 + 0.5 * r * u * u + p) / r for r, p in ((rL, pL), (rR, pR))]
+    sL, sR = np.sqrt(rL), np.sqrt(rR)
+    ch = np.sqrt(gm1 * ((sL * H[0] + sR * H[1]) / (sL + sR) - 0.5 * u * u))
+    SL = np.minimum(u - c, u - ch)
+    SR = np.maximum(u + np.sqrt(gamma * pR / rR), u + ch)
+    S = (rR * u * (SR - u) - rL * u * (SL - u) + (pL - pR)) / (rR * (SR - u) - rL * (SL - u))
+    assert ((SR < 0) & (S >= 0)).sum() >= 3
+    kw = dict(scheme="MEG6")
+    o, s = orc.Oracle(prob, **kw), api.Solver.from_problem(prob, fma_sweep=fma, **kw)
+    # (fused multiply-adds: rounding only)
+    assert rel_err(s.rhs(to_dev(prob["U"])), o.rhs(prob["U"])) <= (1e-9 if fma else 1e-13)
