@@ -300,6 +300,10 @@ __device__ __forceinline__ long long kmin(long long a, long long b) { return a <
 __device__ __forceinline__ long long kmax(long long a, long long b) { return a > b ? a : b; }
 __device__ __forceinline__ double min_f64(double a, double b) { return order_key(a) < order_key(b) ? a : b; }
 __device__ __forceinline__ double max_f64(double a, double b) { return order_key(a) > order_key(b) ? a : b; }
+__device__ __forceinline__ bool is_nan(double x) {
+  return ((unsigned long long)bits64(x) & 0x7fffffffffffffffull) > 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool is_nan(float x) { return (__float_as_uint(x) & 0x7fffffffu) > 0x7f800000u; }
 // 0 <= x (either zero included, NaN not)
 __device__ __forceinline__ bool nonneg(double x) {
   return (unsigned long long)bits64(x) <= 0x7ff0000000000000ull ||

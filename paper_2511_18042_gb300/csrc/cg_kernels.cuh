@@ -633,12 +633,14 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
   // sensor box; node x of the line is at base + x * stride.
   __shared__ int s_lc[LW][3];
   __shared__ long long s_lq[LW], s_lo[LW];
-  // the line's nodes whose sensor is above the threshold, one bit a node (row
-  // r of the sensor window in bit r): an interface's maximum over its window is
-  // above the threshold where any bit of the window is set
-  __shared__ unsigned s_om[LW][4];
+  // the line's nodes whose sensor is above the threshold, and those whose sensor
+  // is NaN, one bit a node (row r of the sensor window in bit r).  The window's
+  // maximum is formed in order, m = m > o ? m : o, so a NaN discards what came
+  // before it: it is above the threshold where a node behind the last NaN is,
+  // which is where the window's bits of s_om, as a number, exceed those of s_nan
+  __shared__ unsigned s_om[LW][4], s_nan[LW][4];
   static_assert(RO <= 96, "three words of node bits and one read past them");
-  if (tid < LW * 4) s_om[tid >> 2][tid & 3] = 0u;
+  if (tid < LW * 4) s_om[tid >> 2][tid & 3] = s_nan[tid >> 2][tid & 3] = 0u;
   if (tid < LW) {
     const int l = tid;
     int c[3] = {0, 0, 0};
@@ -733,12 +735,14 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
       }
       stn(sW, r, l, RW, w);
     });
-    // sensor window: nodes above the threshold
+    // sensor window: nodes above the threshold, nodes without a value
     const T thr = gconst<T>(q.thr, q.f_thr);
     staged(na + 7, RO, [&](int r, int l) {
       int x = i0 - 4 + r;
-      if (s_lc[l][0] >= 0 && x <= n + 3 && static_cast<const T*>(A.om)[s_lo[l] + (long long)x * os] > thr)
-        atomicOr(&s_om[l][r >> 5], 1u << (r & 31));
+      if (s_lc[l][0] < 0 || x > n + 3) return;
+      const T o = static_cast<const T*>(A.om)[s_lo[l] + (long long)x * os];
+      if (o > thr) atomicOr(&s_om[l][r >> 5], 1u << (r & 31));
+      else if (is_nan(o)) atomicOr(&s_nan[l][r >> 5], 1u << (r & 31));
     });
     __syncthreads();
     // 2. first derivatives along DIR on nodes i0-2 .. i0+TL
@@ -811,8 +815,10 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
     if (use_gbr) {
       // nodes i-w+1 .. i+w of the sensor window, w = q.window <= 4
       const int p0 = a + 4 - q.window;
-      const unsigned wb = __funnelshift_r(s_om[l][p0 >> 5], s_om[l][(p0 >> 5) + 1], p0 & 31);
-      const bool disc = (wb & ((1u << (2 * q.window)) - 1u)) != 0u;
+      const unsigned wm = (1u << (2 * q.window)) - 1u;
+      const unsigned wb = __funnelshift_r(s_om[l][p0 >> 5], s_om[l][(p0 >> 5) + 1], p0 & 31) & wm;
+      bool disc = wb != 0u;
+      if (disc) disc = wb > (__funnelshift_r(s_nan[l][p0 >> 5], s_nan[l][(p0 >> 5) + 1], p0 & 31) & wm);
       T xi[3] = {T(0), T(0), T(0)};
       if (!CART) {
         long long pq = plin(g, c[0], c[1], c[2]);

@@ -52,3 +52,21 @@ def test_contact_right_of_the_right_wave(orc, api, gamma, fma):
     o, s = orc.Oracle(prob, **kw), api.Solver.from_problem(prob, fma_sweep=fma, **kw)
     # (fused multiply-adds: rounding only)
     assert rel_err(s.rhs(to_dev(prob["U"])), o.rhs(prob["U"])) <= (1e-9 if fma else 1e-13)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("at", [(16, 32), (16, 44), (16, 56)])
+def test_sensor_window_with_a_nan(orc, api, at, precision):
+    """A node without a value: the nodes whose stencil does not hold it keep
+    theirs.  The window's maximum is taken in order and a comparison with NaN
+    is false, so a NaN discards what came before it."""
+    prob = inputs.triple_point(96, 64)
+    U = orc.Oracle(prob, scheme="MEG6").advance(prob["U"], nsteps=12)[0]
+    U[:, at[1], at[0]] = np.nan
+    kw = dict(scheme="MEG6")
+    Ro = orc.Oracle(prob, **kw).rhs(U)
+    Rg = api.Solver.from_problem(prob, precision=precision, **kw).rhs(to_dev(U)).cpu().numpy()
+    assert np.array_equal(np.isfinite(Rg), np.isfinite(Ro))
+    ok = np.isfinite(Ro).all(axis=0)
+    assert 0 < (~ok).sum() < ok.size // 4
+    assert rel_err(Rg[:, ok], Ro[:, ok]) <= (1e-3 if precision else 1e-13)
