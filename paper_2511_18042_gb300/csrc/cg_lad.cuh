@@ -392,8 +392,10 @@ __global__ void __launch_bounds__(256) k_gauss2_tile(DevGrid g, const T* __restr
   if (guard && *guard != want) return;
   const T A0 = T(3565.0 / 10368.0), A1 = T(3091.0 / 12960.0), A2 = T(1997.0 / 25920.0), A3 = T(149.0 / 12960.0),
           A4 = T(107.0 / 103680.0);
-  const int lx = threadIdx.x % GT_X, x = (int)blockIdx.x * GT_X + lx, y0 = (int)blockIdx.y * GT_Y;
   const int n0 = g.n[0], n1 = g.n[1];
+  const int lx = threadIdx.x % GT_X, x = (int)blockIdx.x * GT_X + lx;
+  const int y0 = ((int)blockIdx.y + (int)blockIdx.z * (int)gridDim.y) * GT_Y;  // rows past 65535 tiles are folded into z
+  if (y0 >= n1) return;
   if (x < n0) {
     for (int r = threadIdx.x / GT_X; r < R && y0 - 4 + r < n1 + 4; r += 256 / GT_X) {
       const long long row = scalar_src(g, 0, y0 - 4 + r, 0);  // node 0 of the row (the boundary rules are separable)

@@ -143,7 +143,8 @@ static int lad_coeffs_run(cg_solver* s, int dkind, cudaStream_t st, const int* g
   }
   s->launches += 2;
   if constexpr (gauss2) {
-    const dim3 grid((unsigned)((s->dg.n[0] + GT_X - 1) / GT_X), (unsigned)((s->dg.n[1] + GT_Y - 1) / GT_Y));
+    const unsigned ty = (unsigned)((s->dg.n[1] + GT_Y - 1) / GT_Y), gy = std::min(ty, 65535u);
+    const dim3 grid((unsigned)((s->dg.n[0] + GT_X - 1) / GT_X), gy, (ty + gy - 1) / gy);
     k_gauss2_tile<T><<<grid, 256, 0, st>>>(s->dg, bt[1], kp[1], bt[0], kp[0], guard, want);
     s->launches++;
     return CG_OK;
