@@ -681,7 +681,7 @@ static GbrCfg gbr_cfg(const cg_solver* s) {
   GbrCfg q;
   q.gamma = s->p.gamma;
   q.gm1 = s->p.gamma - 1.0;
-  q.thr = s->p.sensor_thresh;
+  q.thr = std::isnan(s->p.sensor_thresh) ? INFINITY : s->p.sensor_thresh;  // nothing is above either
   q.eps = s->p.mp_eps;
   q.alpha = s->p.mp_alpha;
   q.window = s->p.omega_window;

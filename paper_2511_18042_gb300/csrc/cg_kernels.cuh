@@ -633,11 +633,11 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
   // sensor box; node x of the line is at base + x * stride.
   __shared__ int s_lc[LW][3];
   __shared__ long long s_lq[LW], s_lo[LW];
-  // the line's nodes whose sensor is above the threshold, and those whose sensor
-  // is NaN, one bit a node (row r of the sensor window in bit r).  The window's
-  // maximum is formed in order, m = m > o ? m : o, so a NaN discards what came
-  // before it: it is above the threshold where a node behind the last NaN is,
-  // which is where the window's bits of s_om, as a number, exceed those of s_nan
+  // the line's nodes whose sensor is above the threshold or NaN, and the NaN ones
+  // among them, one bit a node (row r of the sensor window in bit r).  The
+  // window's maximum is formed in order, m = m > o ? m : o, so a NaN discards what
+  // came before it: it is above the threshold where a node behind the last NaN is,
+  // which is where the other bits of s_om, as a number, exceed those of s_nan
   __shared__ unsigned s_om[LW][4], s_nan[LW][4];
   static_assert(RO <= 96, "three words of node bits and one read past them");
   if (tid < LW * 4) s_om[tid >> 2][tid & 3] = s_nan[tid >> 2][tid & 3] = 0u;
@@ -741,8 +741,10 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
       int x = i0 - 4 + r;
       if (s_lc[l][0] < 0 || x > n + 3) return;
       const T o = static_cast<const T*>(A.om)[s_lo[l] + (long long)x * os];
-      if (o > thr) atomicOr(&s_om[l][r >> 5], 1u << (r & 31));
-      else if (is_nan(o)) atomicOr(&s_nan[l][r >> 5], 1u << (r & 31));
+      if (!(o <= thr)) {
+        atomicOr(&s_om[l][r >> 5], 1u << (r & 31));
+        if (is_nan(o)) atomicOr(&s_nan[l][r >> 5], 1u << (r & 31));
+      }
     });
     __syncthreads();
     // 2. first derivatives along DIR on nodes i0-2 .. i0+TL
@@ -818,7 +820,10 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
       const unsigned wm = (1u << (2 * q.window)) - 1u;
       const unsigned wb = __funnelshift_r(s_om[l][p0 >> 5], s_om[l][(p0 >> 5) + 1], p0 & 31) & wm;
       bool disc = wb != 0u;
-      if (disc) disc = wb > (__funnelshift_r(s_nan[l][p0 >> 5], s_nan[l][(p0 >> 5) + 1], p0 & 31) & wm);
+      if (disc) {
+        const unsigned nb = __funnelshift_r(s_nan[l][p0 >> 5], s_nan[l][(p0 >> 5) + 1], p0 & 31) & wm;
+        disc = (wb & ~nb) > nb;
+      }
       T xi[3] = {T(0), T(0), T(0)};
       if (!CART) {
         long long pq = plin(g, c[0], c[1], c[2]);

@@ -70,3 +70,14 @@ def test_sensor_window_with_a_nan(orc, api, at, precision):
     ok = np.isfinite(Ro).all(axis=0)
     assert 0 < (~ok).sum() < ok.size // 4
     assert rel_err(Rg[:, ok], Ro[:, ok]) <= (1e-3 if precision else 1e-13)
+
+
+@pytest.mark.parametrize("thresh", [float("nan"), float("inf"), -1.0])
+def test_sensor_thresholds_out_of_the_ordinary(orc, api, thresh):
+    """No node is above NaN or infinity (the linear reconstruction everywhere);
+    every node is above a negative threshold."""
+    prob = inputs.triple_point(96, 64)
+    U = orc.Oracle(prob, scheme="MEG6").advance(prob["U"], nsteps=12)[0]
+    kw = dict(scheme="MEG6", sensor_thresh=thresh)
+    Ro = orc.Oracle(prob, **kw).rhs(U)
+    assert rel_err(api.Solver.from_problem(prob, **kw).rhs(to_dev(U)), Ro) <= 1e-13
