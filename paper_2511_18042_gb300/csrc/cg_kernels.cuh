@@ -564,6 +564,37 @@ static __device__ __noinline__ void gbr_flux_ieee(const GbrCfg& q, const DevGrid
   for (int v = 0; v < NV; ++v) io[v] = F[v];
 }
 
+// The interfaces that gbr_flux_f64 with products on the integer pipes does not
+// take: the same form with plain products, whose factors may have any size, then
+// the IEEE form.  Behind a call: most flows never run it, but compact gradients
+// decay by a constant factor a row (0.268) beside a jump into gas at rest, and
+// pass through 2^-400 to the smallest double on rows 210 to 570 from it.  There
+// (s_small in the sweep) it is taken at once.  MIG4 step of the triple point
+// 1792 x 768, a fifth of the x and half of the y interfaces there: 6.57 ms with
+// the IEEE form after the refused one, 5.26 with this form after it, 4.53 with
+// this form at once (MEG6: 3.76).
+template <int ND, bool CART, int DIR, int LW, int UNIT>
+static __device__ __noinline__ void gbr_flux_rare(const GbrCfg& q, const DevGrid& g, const double* sW, const double* sD,
+                                                  const double* sH, int a, int l, bool disc, double* io) {
+  if constexpr (UNIT == 0) {
+    constexpr int NV = ND + 2, RW = SWEEP_TL + 9, RD = SWEEP_TL + 3, RDD = SWEEP_TL + 1;
+    auto ld = [&](const double* b, int r, int rows, double* w) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) w[v] = b[DIR == 0 ? (v * LW + l) * rows + r : (v * rows + r) * LW + l];
+    };
+    const double xi[3] = {io[0], io[1], io[2]};
+    double F[NV];
+    if (gbr_flux_f64<ND, CART, DIR, false, false>(
+            q, g, [&](int j, double* w) { ld(sW, a + 2 + j, RW, w); }, [&](int j, double* w) { ld(sD, a + 1 + j, RD, w); },
+            [&](int j, double* w) { ld(sH, a + j, RDD, w); }, disc, xi, F)) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) io[v] = F[v];
+      return;
+    }
+  }
+  gbr_flux_ieee<ND, CART, DIR, LW>(q, g, sW, sD, sH, a, l, disc, io);
+}
+
 // T = double: FP64 form; T = float: mixed form (FP32 reconstruction and
 // fluxes from FP64 primitives; FP64 flux differences, residual and RK update).
 // UNIT tags the translation unit that compiles the kernel (0: FP64 without
@@ -640,7 +671,14 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
   // which is where the other bits of s_om, as a number, exceed those of s_nan
   __shared__ unsigned s_om[LW][4], s_nan[LW][4];
   static_assert(RO <= 96, "three words of node bits and one read past them");
-  if (tid < LW * 4) s_om[tid >> 2][tid & 3] = s_nan[tid >> 2][tid & 3] = 0u;
+  // FP64: rows of the first derivatives (row r in bit r) with a value too small for
+  // products on the integer pipes (gbr_flux_rare)
+  constexpr bool SMALL = UNIT == 0;
+  __shared__ unsigned s_small[SMALL ? LW : 1][4];
+  if (tid < LW * 4) {
+    s_om[tid >> 2][tid & 3] = s_nan[tid >> 2][tid & 3] = 0u;
+    if (SMALL) s_small[tid >> 2][tid & 3] = 0u;
+  }
   if (tid < LW) {
     const int l = tid;
     int c[3] = {0, 0, 0};
@@ -774,6 +812,12 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
 #pragma unroll
         for (int v = 0; v < NV; ++v)
           d[v] = ok ? (MIX ? T(A.Gdf[A.gdLB.at(v, x, c)]) : T(A.Gd[A.gdLB.at(v, x, c)])) : T(0);
+        if constexpr (SMALL) {
+          F64Range R;
+#pragma unroll
+          for (int v = 0; v < NV; ++v) R.any0(d[v]);
+          if (!R.ok()) atomicOr(&s_small[l][r >> 5], 1u << (r & 31));
+        }
       }
       stn(sD, r, l, RD, d);
     });
@@ -841,13 +885,16 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
         }
         gbr_flux<ND, CART, DIR, T>(q, g, Wst, Wd, Wdd, disc, xi, F);
       } else {
-        const bool good = gbr_flux_f64<ND, CART, DIR, UN, UNIT == 0>(
-            q, g, [&](int j, double* w) { ldn(sW, a + 2 + j, l, RW, w); },
-            [&](int j, double* w) { ldn(sD, a + 1 + j, l, RD, w); }, [&](int j, double* w) { ldn(sDD, a + j, l, RDD, w); },
-            disc, xi, F);
+        // derivatives of nodes i-1 .. i+2 (rows a .. a+3): the first and second ones the flux reads
+        bool good = false;
+        if (!SMALL || !A.compact || (__funnelshift_r(s_small[l][a >> 5], s_small[l][(a >> 5) + 1], a & 31) & 15u) == 0u)
+          good = gbr_flux_f64<ND, CART, DIR, UN, UNIT == 0>(
+              q, g, [&](int j, double* w) { ldn(sW, a + 2 + j, l, RW, w); },
+              [&](int j, double* w) { ldn(sD, a + 1 + j, l, RD, w); },
+              [&](int j, double* w) { ldn(sDD, a + j, l, RDD, w); }, disc, xi, F);
         if (!good) {
           double io[5] = {xi[0], xi[1], xi[2], 0.0, 0.0};
-          gbr_flux_ieee<ND, CART, DIR, LW>(q, g, sW, sD, sDD, a, l, disc, io);
+          gbr_flux_rare<ND, CART, DIR, LW, UNIT>(q, g, sW, sD, sDD, a, l, disc, io);
 #pragma unroll
           for (int v = 0; v < NV; ++v) F[v] = io[v];
         }
