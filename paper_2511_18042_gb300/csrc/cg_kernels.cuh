@@ -410,6 +410,10 @@ __global__ void k_omega(DevGrid g, const T* __restrict__ W, const T* __restrict_
 // (3D FP64 at three blocks an SM, 85 registers: 1.80 ms a step of the 3D ramp
 // 256 x 96 x 64 instead of 1.89 at two.)
 constexpr int OMT_X = 32, OMT_Y = 8, OMT_H = 3;
+template <int ND, typename T>
+__host__ __device__ constexpr int omega_tile_smem() {
+  return (int)sizeof(T) * (1 + ND) * (OMT_X + 2 * OMT_H) * (OMT_Y + 2 * OMT_H);
+}
 template <int ND, bool CART, typename T>
 __device__ __forceinline__ void k_omega_tile_body(const VBlock& vb, const DevGrid& g, const T* __restrict__ W,
                                                   T* __restrict__ om, const Box& ob) {
@@ -521,20 +525,31 @@ __host__ __device__ constexpr int sweep_smem_doubles() {
 }
 
 // Blocks per SM the register budget is sized for (256 threads a block):
-// * FP64, Cartesian: three (80 registers, up to 40 bytes a thread spill).  The
-//   products on the integer pipes make long dependent chains: the MEG6 sweeps
-//   of the triple point take 4.20 ms a step at two blocks, 3.77 at three and at
-//   four; blocks of 128 threads were slower (4.6: more distinct code in flight).
+// * FP64, Cartesian: three (80 registers).  The products on the integer pipes
+//   make long dependent chains: the MEG6 sweeps of the triple point take 4.20 ms
+//   a step at two blocks, 3.77 at three and at four; blocks of 128 threads were
+//   slower (4.6: more distinct code in flight).  Spills: up to 60 bytes a thread
+//   in 1D and 2D, 70-110 in 3D.
+//   1D and 2D: two where the shared memory does not hold three blocks.  A MEG6
+//   step of the triple point with 16 lines (one block) takes 4.28 ms instead of
+//   4.34; FP64 steps of 48 grids by the persistent stage (more_smem: its sensor
+//   tiles) with 8 lines 11.0 instead of 11.4.
+//   3D: three although 8 lines (86 KB) leave two blocks: 80 registers are the
+//   faster form at that residency too, a MEG6 step of 130^3 15.6 ms instead of
+//   16.0 (16 lines, one block: 17.6 and 18.0).
 // * FP64, curvilinear: two (128 registers): at three the 3D ramp's sweeps,
 //   which spill there, took 14.7 ms a step instead of 14.4.
 // * 1D/2D FP32: four (64 registers; up to 40 bytes a thread spill).  The
 //   kernel is latency-bound at two blocks, 16 warps an SM: four took the
 //   triple point's mixed MEG6 step from 1.24 to 1.02 ms.
-// * 3D FP32: three (85 registers; up to 112 bytes a thread spill): on the 3D
+// * 3D FP32: three; 1.5x the arithmetic per value.  Three runs 4-6 % and on the
 //   ramp 10-15 % faster than two.
-template <int ND, bool CART, typename T>
-__host__ __device__ constexpr int sweep_min_blocks() {
-  return sizeof(T) == 8 ? (CART ? 3 : 2) : (ND <= 2 ? 4 : 3);
+template <int ND, bool CART, typename T, int LW>
+__host__ __device__ constexpr int sweep_min_blocks(int more_smem = 0) {
+  if (sizeof(T) == 4) return ND <= 2 ? 4 : 3;
+  // beside the tile: the lines' tables (under 2 KB) and the 1 KB the system takes, of 228 KB an SM
+  const int smem = (int)sizeof(T) * sweep_smem_doubles<ND, LW>() + more_smem + 3 * 1024;
+  return CART && (ND == 3 || 3 * smem <= 228 * 1024) ? 3 : 2;
 }
 
 // The IEEE form of one interface flux of the FP64 sweep, from the staged tile:
@@ -953,7 +968,7 @@ __device__ __forceinline__ void k_gbr_sweep_body(const VBlock& vb, const DevGrid
 }
 
 template <int ND, int DIR, bool CART, bool COMPACT, typename T, int LW, int UNIT, bool UN>
-__global__ void __launch_bounds__(SWEEP_THREADS, sweep_min_blocks<ND, CART, T>())
+__global__ void __launch_bounds__(SWEEP_THREADS, sweep_min_blocks<ND, CART, T, LW>())
     k_gbr_sweep(const __grid_constant__ DevGrid g, const __grid_constant__ GbrCfg q, const __grid_constant__ StageArgs A) {
   k_gbr_sweep_body<ND, DIR, CART, COMPACT, T, LW, UNIT, UN>(hw_block(), g, q, A);
 }

@@ -79,7 +79,7 @@ int launch_dir(int lw, bool cart, bool compact, const DevGrid& g, const GbrCfg& 
 // Batched sweep: block b of the launch belongs to the grid m = mem[b]
 // (off[m] <= b < off[m + 1]) and is that grid's tile (b - off[m]).
 template <int DIR, int LW>
-__global__ void __launch_bounds__(256, sweep_min_blocks<SND, true, ST>())
+__global__ void __launch_bounds__(256, sweep_min_blocks<SND, true, ST, LW>())
     k_gbr_sweep_batched(const SweepJob* __restrict__ jobs, const long long* __restrict__ off,
                         const int* __restrict__ mem) {
   const long long b = blockIdx.x;
@@ -184,7 +184,8 @@ __device__ __forceinline__ void run_sweep_phase(const PhaseRef& K) {
 // second direction's node fluxes buffers of their own), so no SM can hold a
 // stale line of it.
 template <int LW0, int LW1>
-__global__ void __launch_bounds__(256, sweep_min_blocks<SND, true, ST>()) k_stage_persistent(PersistentStage P) {
+__global__ void __launch_bounds__(256, sweep_min_blocks<SND, true, ST, (LW0 > LW1 ? LW0 : LW1)>(omega_tile_smem<SND, ST>()))
+    k_stage_persistent(PersistentStage P) {
   using T = ST;
 #define CGK_BARRIER() \
   if (!grid_barrier(P.bar, P.err, P.expect)) return
