@@ -653,7 +653,7 @@ struct TimedRegion {
 // ---------------------------------------------------------------- launches
 template <int ND, bool CART, bool COMPACT>
 static void launch_omega(cg_solver* s, cudaStream_t st, const int* guard, int want) {
-  long long tot = s->omBox.size();
+  [[maybe_unused]] const long long tot = s->omBox.size();
   if constexpr (ND >= 2 && !COMPACT) {
     const Box& ob = s->omBox;
     dim3 grid((unsigned)((ob.ext[0] + OMT_X - 1) / OMT_X), (unsigned)((ob.ext[1] + OMT_Y - 1) / OMT_Y),
@@ -663,17 +663,16 @@ static void launch_omega(cg_solver* s, cudaStream_t st, const int* guard, int wa
           s->dg, reinterpret_cast<const float*>(s->W), reinterpret_cast<float*>(s->om), ob, guard, want);
     else
       k_omega_tile<ND, CART, double><<<grid, dim3(OMT_X, OMT_Y), 0, st>>>(s->dg, s->W, s->om, ob, guard, want);
-    s->launches++;
-    return;
+  } else {
+    if (s->p.precision == CG_MIXED)
+      k_omega<ND, CART, COMPACT, float><<<grid_blocks(tot, 128), 128, 0, st>>>(
+          s->dg, reinterpret_cast<const float*>(s->W), reinterpret_cast<const float*>(s->G[0]),
+          reinterpret_cast<const float*>(s->G[1]), reinterpret_cast<const float*>(s->G[2]), s->gdLB[0], s->gdLB[1],
+          s->gdLB[2], reinterpret_cast<float*>(s->om), s->omBox, guard, want);
+    else
+      k_omega<ND, CART, COMPACT, double><<<grid_blocks(tot, 128), 128, 0, st>>>(
+          s->dg, s->W, s->G[0], s->G[1], s->G[2], s->gdLB[0], s->gdLB[1], s->gdLB[2], s->om, s->omBox, guard, want);
   }
-  if (s->p.precision == CG_MIXED)
-    k_omega<ND, CART, COMPACT, float><<<grid_blocks(tot, 128), 128, 0, st>>>(
-        s->dg, reinterpret_cast<const float*>(s->W), reinterpret_cast<const float*>(s->G[0]),
-        reinterpret_cast<const float*>(s->G[1]), reinterpret_cast<const float*>(s->G[2]), s->gdLB[0], s->gdLB[1],
-        s->gdLB[2], reinterpret_cast<float*>(s->om), s->omBox, guard, want);
-  else
-    k_omega<ND, CART, COMPACT, double><<<grid_blocks(tot, 128), 128, 0, st>>>(
-        s->dg, s->W, s->G[0], s->G[1], s->G[2], s->gdLB[0], s->gdLB[1], s->gdLB[2], s->om, s->omBox, guard, want);
   s->launches++;
 }
 

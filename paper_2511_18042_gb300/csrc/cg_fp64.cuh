@@ -19,9 +19,15 @@
 // operation returns, which the tests compare on hard operands.  (Newton's
 // iteration and exact remainders: Markstein, IBM J. Res. Dev. 34 (1990) 111.)
 //
-// Operands: magnitudes 2^-400 .. 2^400, numerators also zero.  A caller
-// collects the range tests of its operands (F64Range) and repeats its whole
-// evaluation with IEEE operations when one fails, or uses the checked forms
+// Operands: what div_by, rcp_by, sqrt_ranged and mul_int need is normal
+// operands (a numerator or a second factor also zero) and a normal result:
+// their exponents are sums and differences in one integer word, without a
+// check.  The range tests (F64Range) bound the operands they see by 2^-400 ..
+// 2^400, so that a few may be combined before the next test; the longest chain,
+// the reciprocal of c^2 = gamma p / rho through its root (gamma within 2^+-100,
+// p and rho tested), stays within 2^+-905.  A
+// caller collects the tests and repeats its whole evaluation with plain
+// products or IEEE operations when one fails, or uses the checked forms
 // (div_f64, sqrt_f64), which take the IEEE operation for such an operand.
 // NaN, infinities, subnormals, zero denominators and negative radicands fail
 // the test.
@@ -350,25 +356,6 @@ __device__ __forceinline__ double div_t(double a, double b) { return div_f64(a, 
 __device__ __forceinline__ float div_t(float a, float b) { return a / b; }
 __device__ __forceinline__ double sqrt_t(double x) { return sqrt_f64(x); }
 __device__ __forceinline__ float sqrt_t(float x) { return sqrtf(x); }
-// a/b and c/b
-__device__ __forceinline__ void div2_t(double a, double c, double b, double& qa, double& qc) {
-  F64Range R;
-  R.any0(a);
-  R.any0(c);
-  R.any(b);
-  if (R.ok()) {
-    const Divisor D = divisor(b);
-    qa = div_by(a, D);
-    qc = div_by(c, D);
-  } else {
-    qa = div_ieee(a, b);
-    qc = div_ieee(c, b);
-  }
-}
-__device__ __forceinline__ void div2_t(float a, float c, float b, float& qa, float& qc) {
-  qa = a / b;
-  qc = c / b;
-}
 // 1/x
 __device__ __forceinline__ double rcp_f64(double x) {
   F64Range R;

@@ -320,6 +320,7 @@ __device__ __forceinline__ double sdot_f64(const PR& P, const double* a, const d
 template <int ND, bool CART, int DIR, bool UN, class PR>
 __device__ __forceinline__ void to_char_f64(const PR& P, const Frame<ND, double>& f, const double* w,
                                             double* c) {
+  static_assert(!UN || ND <= 2, "exact unit normals: 1D and 2D");
   constexpr int IP = ND + 1;
   const double un = UN ? by_sign(f.n[DIR], w[1 + DIR]) : sdot_f64<ND, CART, DIR, 0>(P, f.n, w + 1);
   const double a = P.kz(f.ha, w[IP]), b = P.kz(f.hb, un);
@@ -327,10 +328,8 @@ __device__ __forceinline__ void to_char_f64(const PR& P, const Frame<ND, double>
   c[1] = __fma_rn(-2.0, a, w[0]);
   c[IP] = a + b;
 #pragma unroll
-  for (int m = 0; m < ND; ++m) {
+  for (int m = 0; m < ND; ++m)
     if (UN && ND >= 2 && frame_nz(CART, ND, DIR, 1, m)) c[2] = by_sign(f.t1[m], w[1 + m]);
-    if (UN && ND == 3 && frame_nz(CART, ND, DIR, 2, m)) c[3] = by_sign(f.t2[m], w[1 + m]);
-  }
   if (!UN && ND >= 2) c[2] = sdot_f64<ND, CART, DIR, 1>(P, f.t1, w + 1);
   if (!UN && ND == 3) c[3] = sdot_f64<ND, CART, DIR, 2>(P, f.t2, w + 1);
 }
@@ -348,8 +347,7 @@ __device__ __forceinline__ void from_char_f64(const PR& P, const Frame<ND, doubl
   for (int m = 0; m < ND; ++m) {
     if (UN) {
       if (m == DIR) w[1 + m] = by_sign(f.n[m], un);
-      else if (ND >= 2 && frame_nz(CART, ND, DIR, 1, m)) w[1 + m] = by_sign(f.t1[m], c[2]);
-      else w[1 + m] = by_sign(f.t2[m], c[3]);
+      else w[1 + m] = by_sign(f.t1[m], c[2]);
       continue;
     }
     auto t = [&](double a, double b) { return CART ? P.kz(a, b) : P.zz(a, b); };
