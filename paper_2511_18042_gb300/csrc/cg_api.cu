@@ -681,7 +681,7 @@ static GbrCfg gbr_cfg(const cg_solver* s) {
   q.gamma = s->p.gamma;
   q.gm1 = s->p.gamma - 1.0;
   q.thr = std::isnan(s->p.sensor_thresh) ? INFINITY : s->p.sensor_thresh;  // nothing is above either
-  q.eps = s->p.mp_eps;
+  q.eps = s->p.mp_eps + 0.0;  // -0 as 0 (the FP64 sweep compares bit patterns)
   q.alpha = s->p.mp_alpha;
   q.window = s->p.omega_window;
   q.f_gamma = (float)q.gamma;

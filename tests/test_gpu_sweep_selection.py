@@ -81,3 +81,12 @@ def test_sensor_thresholds_out_of_the_ordinary(orc, api, thresh):
     kw = dict(scheme="MEG6", sensor_thresh=thresh)
     Ro = orc.Oracle(prob, **kw).rhs(U)
     assert rel_err(api.Solver.from_problem(prob, **kw).rhs(to_dev(U)), Ro) <= 1e-13
+
+
+@pytest.mark.parametrize("eps", [0.0, -0.0])
+def test_mp_tolerance_of_either_zero(orc, api, eps):
+    prob = inputs.triple_point(96, 64)
+    U = orc.Oracle(prob, scheme="MEG6").advance(prob["U"], nsteps=12)[0]
+    kw = dict(scheme="MEG6", mp_eps=eps)
+    Ro = orc.Oracle(prob, **kw).rhs(U)
+    assert rel_err(api.Solver.from_problem(prob, **kw).rhs(to_dev(U)), Ro) <= 1e-13
