@@ -253,12 +253,13 @@ __device__ __forceinline__ void gbr_flux(const GbrCfg& q, const DevGrid& g, cons
 //   * on a Cartesian grid whose unit normals are exactly 1 (UN) no
 //     multiplication by them.
 // Measured (triple point 1792 x 768, MEG6, with the staging and the epilogue):
-// FP64 instructions an interface 569 -> 272 without the products on the integer
-// pipes, about 190 with them; the sweep 1.51 -> 0.76 -> 0.63 ms a launch, the
-// whole step 9.98 -> 5.23 -> 4.26 ms.
+// FP64 instructions an interface 569 -> 278 without the products on the integer
+// pipes, 181 to 200 with them; the sweep 1.51 -> 0.76 -> 0.61 ms a launch, the
+// whole step 9.98 -> 5.23 -> 4.19 ms.
 // Returns false where an operand is out of the range of these forms (a state
 // that is not positive, NaN, extreme magnitudes): the caller then repeats the
-// interface with gbr_flux.
+// interface, with plain products if it had them on the integer pipes, or with
+// gbr_flux.
 // (mp5's value; the range tests of its operands go to R)
 __device__ __forceinline__ double mp5_f64(double um2, double um1, double u0, double up1, double up2, double alpha,
                                           double eps, F64Range& R) {
@@ -469,10 +470,10 @@ template <int ND, bool CART, int DIR, bool UN, bool IM, class FW, class FD, clas
 __device__ __forceinline__ bool gbr_flux_f64(const GbrCfg& q, const DevGrid& g, FW ldW, FD ldD, FH ldH, bool disc,
                                              const double* xi, double* F) {
   constexpr int NV = ND + 2, IP = ND + 1;
+  if (!q.f64_fast) return false;  // at once: the caller's IEEE form is all that is paid
   F64Range R;
   using PR = std::conditional_t<IM, F64Products, PlainProducts>;
   const PR P = make_products<PR>(R);
-  if (!q.f64_fast) R.see(~0u);
   Frame<ND, double> fr;
   double g2, gg, ig2, xl[3];
   if (CART) {
