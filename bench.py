@@ -55,11 +55,15 @@ METRIC = "cell-updates/s per scheme & % HBM roofline; batched solves/s, p50/p99 
 # the flop-counting build of the oracle on the developed triple-point state:
 # profiles/flops_triple_point_1792x768.md (oracle/count_flops.py).
 SWEEP_FLOP_PER_IFACE = 524.8
-# dram read + write per launch (mean of x and y) of the sweep form the roofline times,
-# from its ncu capture (profiles/); None until the current kernel has been captured
 # the bounded sample of the triple point on which the CPU oracle is timed
 CPU_SAMPLE = (896, 384)
-SWEEP_TRAFFIC_BYTES = {"exact": 118.0e6, "contracted": 140.2e6}
+# dram read + write per launch and instructions issued to the FP64 pipe per
+# interface (mean of the x and y launches of the bench state's MEG6 step, the
+# default tiles) of each sweep form, from its ncu capture
+# (profiles/sweep_meg6_integer_pipes_1792x768.md); None until the current kernel
+# has been captured
+SWEEP_TRAFFIC_BYTES = {"exact": 130.2e6, "contracted": 131.2e6}
+SWEEP_FP64_INSTR_PER_IFACE = {"exact": 180.9, "contracted": 210.7}
 ROOFLINE_FORM = "exact"  # the library default (fma_sweep = 0)
 FP64_PEAK_DERIVED_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12  # SMs x DFMA/clk x 2 flop x max clock (context only)
 HBM_BYTES_PER_CELL_STEP = 256.0  # minimal-traffic model, FP64 state, nv = 4, uniform grid
@@ -668,9 +672,10 @@ def _sweep_ms(api, torch, grid, base, dev, args, form):
 
 def sweep_roofline(api, torch, grid, base, dev, args, peaks):
     """FP64 roofline of the dominant kernel, the MEG6 interface sweep, in the
-    library's default (exact) form: algorithmic flop per interface (oracle
-    count) x interfaces per launch / measured launch time, against the
-    measured FP64 FMA peak; the opt-in FMA form beside it."""
+    library's default (exact) form: FP64-pipe instructions per interface (ncu)
+    x interfaces per launch / measured launch time, against the measured FP64
+    FMA peak, and the algorithmic rate (oracle's operation count) beside it;
+    the same for the opt-in FMA form."""
     ifaces = ((NX + 1) * NY + NX * (NY + 1)) / 2.0  # algorithmic interfaces per sweep launch (x, y average)
     peak = peaks["fp64_tflops"]
     avg_ms, n, tile = _sweep_ms(api, torch, grid, base, dev, args, ROOFLINE_FORM)
@@ -682,18 +687,29 @@ def sweep_roofline(api, torch, grid, base, dev, args, peaks):
             "launch_ms": avg_ms, "launches": n, "ifaces_per_launch": ifaces,
             "traffic": SWEEP_TRAFFIC_BYTES[ROOFLINE_FORM], "form": ROOFLINE_FORM,
             "tile_lines": list(tile)}
-    ach = SWEEP_FLOP_PER_IFACE * ifaces / (avg_ms * 1e-3) / 1e12
-    roof.update({"achieved": ach, "frac": ach / peak, "algorithmic_flop_per_iface": SWEEP_FLOP_PER_IFACE,
+    roof.update(_sweep_rates(ROOFLINE_FORM, ifaces, avg_ms, peak))
+    roof.update({"algorithmic_flop_per_iface": SWEEP_FLOP_PER_IFACE,
                  "flop_source": "oracle operation count (profiles/flops_triple_point_1792x768.md)",
-                 "frac_note": "divisions, roots, comparisons and products with a known factor run on the integer "
-                              "and FP32 pipes: the counted operations per time may exceed the FP64 pipe's peak",
                  "peak_measured": {k: v for k, v in peaks.items() if k != "clocks"}})
     fms, fn, ftile = _sweep_ms(api, torch, grid, base, dev, args, "contracted")
-    fach = SWEEP_FLOP_PER_IFACE * ifaces / (fms * 1e-3) / 1e12
-    roof["fma_sweep"] = {"launch_ms": fms, "launches": fn, "tile_lines": list(ftile), "achieved": fach,
-                         "frac": fach / peak, "traffic": SWEEP_TRAFFIC_BYTES["contracted"],
+    roof["fma_sweep"] = {"launch_ms": fms, "launches": fn, "tile_lines": list(ftile),
+                         "traffic": SWEEP_TRAFFIC_BYTES["contracted"],
                          "note": "opt-in FMA form (fma_sweep = 1): not bitwise; see profiles"}
+    roof["fma_sweep"].update(_sweep_rates("contracted", ifaces, fms, peak))
     return roof
+
+
+def _sweep_rates(form, ifaces, ms, peak):
+    """Rates of one sweep launch.  achieved and frac count what is issued to the
+    FP64 pipe, each instruction as the fused multiply-add it takes the place of;
+    divisions, roots, comparisons and (exact form) products with a known factor
+    run on the integer and FP32 pipes, so the algorithmic rate may exceed the
+    FP64 pipe's peak and has no fraction."""
+    per_s = ifaces / (ms * 1e-3)
+    ach = 2.0 * SWEEP_FP64_INSTR_PER_IFACE[form] * per_s / 1e12
+    return {"achieved": ach, "frac": ach / peak, "fp64_pipe_instr_per_iface": SWEEP_FP64_INSTR_PER_IFACE[form],
+            "frac_note": "FP64-pipe instructions (ncu) x 2 flop per launch time, of the measured FMA peak",
+            "algorithmic_tflops": SWEEP_FLOP_PER_IFACE * per_s / 1e12}
 
 
 def _cpu_model():
